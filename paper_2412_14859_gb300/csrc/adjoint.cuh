@@ -20,68 +20,40 @@
 //                pushes the lg part to where the pull read from, the next kernel A adds the ab
 //                part of the writer as it reads lambda^{n+1}
 // Kernel A recomputes the forward quantities of its tile exactly as the step does (it runs the
-// step's own tile code with this file's epilogue in place of the collision/store).
+// step's own tile code with this file's epilogue in place of the collision and store).
 #pragma once
 
 #include "launch.h"
-#include "step_kernel.cuh"
+#include "pair_tile.cuh"
 
 namespace cgevap {
 
 // Minority fraction product w_r w_b below which the adjoint holds the recoloring direction fixed.
 constexpr double kBulkTrace = 1e-6;
 
-// Pull source of direction i from the cell with slot sl at storage index si (see pull_cell).
+// Pull source of direction i from storage index si (see pull_pairs).
 template <class L>
-__device__ __forceinline__ int pull_source(const Slot& sl, const PlaneOffsets& po, int si, int i) {
-  return si + (L::ca(i) > 0 ? sl.dxm : (L::ca(i) < 0 ? sl.dxp : 0)) +
-         (L::cb(i) > 0 ? sl.dym : (L::cb(i) < 0 ? sl.dyp : 0)) +
-         (L::cm(i) > 0 ? po.dm_lo : (L::cm(i) < 0 ? po.dm_hi : 0));
+__device__ __forceinline__ int pull_source(int4 to, int lo, int hi, int si, int i) {
+  return si + (L::ca(i) > 0 ? to.x : (L::ca(i) < 0 ? to.y : 0)) +
+         (L::cb(i) > 0 ? to.z : (L::cb(i) < 0 ? to.w : 0)) + (L::cm(i) > 0 ? lo : (L::cm(i) < 0 ? hi : 0));
 }
 
-// (1) for one cell: recompute the moments, F and the per-direction terms of collide_store and
-// run them backwards.  fcb: colour-blind sums of the post-exchange populations (rho_r, rho_b
-// given separately); lam: dL/d(f^{r*}, f^{b*}) of this cell;
-// out: lg = dL/dg through this cell's own collision, lF = dL/dF.
-// lam_at(i): lambda^{n+1} of direction i (loaded where it is used); lg_out(i, v): stores lg_i.
+// (1) for one cell: from its moments c, F and the colour-blind sums f of its post-exchange
+// populations, recompute the per-direction terms of collide_pairs and run them backwards.
+// lam_at(i): lambda^{n+1} of direction i (loaded where it is used); out: lg_out(i, v) takes
+// lg_i = dL/dg_i through this cell's own collision, lF = dL/dF.
 template <int Q, class R, class LamAt, class LgOut>
-__device__ __forceinline__ void collide_adjoint(const Physics& ph, const R (&fcb)[Q], R rr, R rb,
-                                                R irho, const R (&rnb)[Q], const LamAt& lam_at,
+__device__ __forceinline__ void collide_adjoint(const Physics& ph, const CellMoments<R>& c0, const R (&f)[Q],
+                                                R irho, R Fa, R Fb, R Fm, const LamAt& lam_at,
                                                 const LgOut& lg_out, R (&lF)[3]) {
   using L = Lattice<Q>;
-  const R rho = rr + rb;
-  const R wr = rr * irho, wb = rb * irho;
-  R f[Q];
-  R ja = R(0), jb = R(0), jm = R(0);
-#pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    f[i] = fcb[i];
-    if (L::ca(i) > 0) ja += f[i];
-    if (L::ca(i) < 0) ja -= f[i];
-    if (L::cb(i) > 0) jb += f[i];
-    if (L::cb(i) < 0) jb -= f[i];
-    if (L::cm(i) > 0) jm += f[i];
-    if (L::cm(i) < 0) jm -= f[i];
-  }
-  const R ua = ja * irho, ub = jb * irho, um = jm * irho;
-  const R uu15 = R(1.5) * (ua * ua + ub * ub + um * um);
+  const R rho = c0.rho, wr = c0.wr, wb = c0.wb, ua = c0.ua, ub = c0.ub, um = c0.um;
+  const R uu15 = c0.uu15, itau = c0.itau, abar = c0.abar;
   const R ir = PHYS(R, ph, inv_tau_r), ib = PHYS(R, ph, inv_tau_b);
-  const R itau = wr * ir + wb * ib;
-  const R abar = wr * PHYS(R, ph, alpha_r) + wb * PHYS(R, ph, alpha_b);
-  R Fa = R(0), Fb = R(0), Fm = R(0);
-#pragma unroll
-  for (int i = 1; i < Q; ++i) {
-    const R t = R(3.0 * L::W(i)) * rnb[i];
-    if (L::ca(i) > 0) Fa += t;
-    if (L::ca(i) < 0) Fa -= t;
-    if (L::cb(i) > 0) Fb += t;
-    if (L::cb(i) < 0) Fb -= t;
-    if (L::cm(i) > 0) Fm += t;
-    if (L::cm(i) < 0) Fm -= t;
-  }
-  const R F2 = Fa * Fa + Fb * Fb + Fm * Fm;
+  R F2 = fma(Fa, Fa, Fm * Fm);
+  if (L::D3) F2 = fma(Fb, Fb, F2);
   R Fn = R(0), iFn = R(0);
-  if (F2 > R(0)) norm_pair<R>(F2, Fn, iFn);
+  if (F2 > R(0)) norm_of(F2, Fn, iFn);
   const R amp = PHYS(R, ph, amp), beta = PHYS(R, ph, beta);
   const R pamp = amp * itau;
   const R rcol = beta * wr * wb;
@@ -273,17 +245,22 @@ struct AdjointEpilogue {
     }
   }
   template <int Q, int S, class R>
-  __device__ __forceinline__ void cell(const StepArgs& A, int /*cell*/, const Slot& sl,
-                                       uint32_t sbits, int m, int si, int /*nimg*/,
-                                       const int (&)[3], const R (&g)[Q], R rr, R rb, R irho,
-                                       R /*e*/, uint32_t /*flags*/, const R (&rnb)[Q],
-                                       int&, R&) const {
+  __device__ __forceinline__ CellMoments<R> before(const StepArgs& A, const R (&f)[Q], R rr, R rb, R irho) const {
+    return cell_moments<Q, R>(A.ph, f, rr, rb, irho);
+  }
+  __device__ __forceinline__ void filled(const StepArgs&, int, uint32_t) const {}
+  template <int Q, int S, class R>
+  __device__ __forceinline__ void cell(const StepArgs& A, int /*cell*/, const int4* own_to, uint32_t sbits,
+                                       const March& pm, int si, const R (&f)[Q], const CellMoments<R>& c,
+                                       R rr, R rb, R irho, R, R, uint32_t /*flags*/,
+                                       const R (&rnb)[Q]) const {
     using L = Lattice<Q>;
     using Vec = typename Storage<S>::vec;
     constexpr int BX = box_x<Q>(), NB = BX * box_y<Q>();
+    const int m = pm.m;
+    const int4 to = *own_to;
     const int ns = A.g.nstore;
     Vec* lout = reinterpret_cast<Vec*>(o.lam_g);
-    const PlaneOffsets po = plane_offsets(A.g, m);
     // this cell's place in the ab box: the thread's own column of the tile (one cell per thread
     // and plane), one in from the halo
     const int bx = (int)threadIdx.x % TX + 1;
@@ -306,11 +283,13 @@ struct AdjointEpilogue {
       v.y = v2.b;
       // element index in 32 bits (a state holds Q nstore < 2^31 vec2)
       const bool bounce = (sbits >> i) & 1u;
-      const int idx = bounce ? opp(i) * ns + si : i * ns + pull_source<L>(sl, po, si, i);
+      const int idx = bounce ? opp(i) * ns + si : i * ns + pull_source<L>(to, pm.lo, pm.hi, si, i);
       lout[idx] = v;
     };
     R lF[3];
-    collide_adjoint<Q, R>(A.ph, g, rr, rb, irho, rnb, lam_at, lg_out, lF);
+    R Fa, Fb, Fm;
+    colour_gradient<Q, R>(rnb, Fa, Fb, Fm);
+    collide_adjoint<Q, R>(A.ph, c, f, irho, Fa, Fb, Fm, lam_at, lg_out, lF);
     R* ax = reinterpret_cast<R*>(o.aux);
     ax[si] = lF[0];
     ax[(size_t)ns + si] = lF[1];
@@ -332,9 +311,9 @@ __global__ void __launch_bounds__(TX* TY, (S == ST_F64 ? 256 : 384) / (TX * TY))
   // lambda columns after the tile's own shared memory (slot i of thread t at i TX TY + t), then
   // the ab box
   constexpr int lam_bytes = Q * TX * TY * (int)sizeof(Vec);
-  unsigned char* const lam0 = dyn_smem + TileSmem<Q, S, TX, TY, 1>::BYTES;
+  unsigned char* const lam0 = dyn_smem + PairSmem<Q, S, TX, TY>::BYTES;
   const Epi E{O, lam0 + threadIdx.x * sizeof(Vec), lam0 + lam_bytes};
-  step_tile<Q, S, TX, TY, 1, Epi>(A, blockIdx.x, blockIdx.y, dyn_smem, n, d, threadIdx.x, -1, E);
+  pair_tile<Q, S, TX, TY, true, true>(A, blockIdx.x, blockIdx.y, dyn_smem, n, d, threadIdx.x, E, CtaSync());
 }
 
 __device__ __forceinline__ void cell_coords(const Geom& g, int cell, int& a, int& b, int& m) {
@@ -362,6 +341,7 @@ __global__ void __launch_bounds__(256)
   uint32_t bits = 0;
   if (!solid_bits<L>(G, sl, p, cell, bits)) return;
   const PlaneOffsets po = plane_offsets(G, m);
+  const int4 to = make_int4(sl.dxm, sl.dxp, sl.dym, sl.dyp);
   const int si = sidx(G, a, b, m);
   const size_t ns = G.nstore;
   const R oa = aux[si], ob = aux[ns + si], om = aux[2 * ns + si];
@@ -370,7 +350,7 @@ __global__ void __launch_bounds__(256)
   for (int i = 1; i < Q; ++i) {
     R t = R(0);
     if (!((bits >> i) & 1u)) {  // x = y - c_i is fluid: its F used rho^N(y) with weight 3 W_i c_i
-      const int src = pull_source<L>(sl, po, si, i);
+      const int src = pull_source<L>(to, po.dm_lo, po.dm_hi, si, i);
       if (L::ca(i)) t += R(L::ca(i)) * __ldg(aux + src);
       if (L::cb(i)) t += R(L::cb(i)) * __ldg(aux + ns + src);
       if (L::cm(i)) t += R(L::cm(i)) * __ldg(aux + 2 * ns + src);

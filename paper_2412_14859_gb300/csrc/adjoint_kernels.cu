@@ -11,7 +11,7 @@ template <int Q, int S, int TX, int TY>
 KernelRef adj_ref() {
   // the tile's shared memory, then the prefetched lambda^{n+1} columns (Q vec per thread), then
   // the box of ab
-  constexpr int smem = TileSmem<Q, S, TX, TY, 1>::BYTES +
+  constexpr int smem = PairSmem<Q, S, TX, TY>::BYTES +
                        Q * TX * TY * (int)sizeof(typename Storage<S>::vec) +
                        AdjointEpilogue<TX, TY>::template box_bytes<Q, S>();
   const void* fn = (const void*)cg_adjoint_local_kernel<Q, S, TX, TY>;

@@ -283,7 +283,7 @@ int launch_one_step(cgevap_sim* s) {
   StepArgs a = step_args(s);
   void* args[] = {&a, s->tmap[s->cur]};
   const KernelRef& k = s->rc_pairs && s->kernel_in.fn ? s->kernel_in : s->kernel;
-  CG_CUDA(s, cudaLaunchKernel(k.fn, dim3(s->ntx * s->nty, s->nchunk), dim3(k.threads), args, k.smem,
+  CG_CUDA(s, cudaLaunchKernel(step_fn(k, a), dim3(s->ntx * s->nty, s->nchunk), dim3(k.threads), args, k.smem,
                               s->stream));
   s->cur ^= 1;
   s->rc_pairs = 0;

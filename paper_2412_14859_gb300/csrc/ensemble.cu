@@ -5,10 +5,9 @@
 // Work list.  A step of a member is split into items: (member, tile, chunk of planes) exactly as
 // the single-lattice step kernel splits it.  A D3Q19 item fills a 128-thread CTA (32 x 4 tile;
 // four CTAs per SM, as the fastest single-lattice step); D2Q9 items are narrower and run G at a
-// time in one CTA, one per group of 128/G threads (row tiles of 128/G cells), with their barrier
-// rounds padded to the longest chunk of the pack.  Members store FP32 or FP64 populations, or
-// all of them FP32 pairs with exact colour masses; a pack holds items of one storage only, so
-// every barrier round of a CTA runs the same code.
+// time in one CTA, one per group of 128/G threads (row tiles of 128/G cells) with a barrier of its
+// own, so the groups march independently.  Members store FP32 or FP64 populations, or
+// all of them FP32 pairs with exact colour masses; a pack holds items of one storage only.
 // CTAs take items (or packs) from a counter, meet at a grid barrier after every step, and fold
 // the per-item ledger partials of each member in item order (deterministic).  Every wait is
 // bounded (4 s by default, settable from the host); a barrier that gives up sets the status
@@ -24,7 +23,7 @@
 #include "../../include/cgevap.h"
 #include "launch.h"
 #include "sim.h"
-#include "step_kernel.cuh"
+#include "pair_tile.cuh"
 
 using namespace cgevap;
 
@@ -103,10 +102,21 @@ constexpr int ens_s32() {
 // Shared memory of one D2Q9 group / one D3Q19 item of storage S.
 template <int G, int S>
 constexpr int ens_group_smem() {
-  return TileSmem<9, S, kEnsThreads / G, 1, 1>::BYTES;
+  return PairSmem<9, S, kEnsThreads / G, 1>::BYTES;
 }
 
-template <int G, int MODE>
+// The barrier of a D2Q9 group of GT threads: a warp, or a named barrier of its own.
+template <int GT>
+struct GroupSyncOf {
+  static_assert(GT == 64, "groups are a warp or 64 threads");
+  using type = PairSync;
+};
+template <>
+struct GroupSyncOf<32> {
+  using type = WarpSync;
+};
+
+template <int G, int MODE, bool GEN>
 __global__ void __launch_bounds__(kEnsThreads, MODE == kEnsF32 || MODE == kEnsF32X ? 4 : 2)
     cg_ensemble_kernel(const __grid_constant__ EnsArgs E) {
   constexpr int NT = kEnsThreads;
@@ -117,6 +127,22 @@ __global__ void __launch_bounds__(kEnsThreads, MODE == kEnsF32 || MODE == kEnsF3
   __shared__ long long gsum_n[NT / 32];
   const int tid = threadIdx.x;
   const int grp = tid / GT, gtid = tid % GT;
+  __shared__ StepArgs args[G];  // of the item, or of each group's
+  // the arguments of item (member j) for this step, copied by nt threads
+  auto load_args = [&](StepArgs& A, int j, int t, int nt) {
+    const EnsMember& M = E.members[j];
+    static_assert(sizeof(StepArgs) % 4 == 0, "copied in words");
+    for (int w = t; w < (int)(sizeof(StepArgs) / 4); w += nt)
+      reinterpret_cast<uint32_t*>(&A)[w] = reinterpret_cast<const uint32_t*>(&M.a)[w];
+  };
+  auto set_buffers = [&](StepArgs& A, int j, int step) {  // one thread, after the copy
+    const EnsMember& M = E.members[j];
+    const int c = (E.cur[j] + step) & 1;
+    A.pin = M.state[c];
+    A.pout = M.state[c ^ 1];
+    A.mask_in = M.mask[c];
+    A.mask_out = M.mask[c ^ 1];
+  };
   for (int step = 0; step < E.nsteps; ++step) {
     const int par = step & 1;
     double* pr = E.part_removed + (size_t)par * E.nitems;
@@ -137,18 +163,15 @@ __global__ void __launch_bounds__(kEnsThreads, MODE == kEnsF32 || MODE == kEnsF3
       double d = 0.0;
       if (w < E.n3) {
         const int4 it = E.items[w];
-        const EnsMember& M = E.members[it.x];
-        StepArgs A = M.a;
-        const int c = (E.cur[it.x] + step) & 1;
-        A.pin = M.state[c];
-        A.pout = M.state[c ^ 1];
-        A.mask_in = M.mask[c];
-        A.mask_out = M.mask[c ^ 1];
-        const bool f64 = MODE == kEnsF64 || (MODE == kEnsMixed && M.storage == ST_F64);
+        load_args(args[0], it.x, tid, NT);
+        __syncthreads();
+        if (tid == 0) set_buffers(args[0], it.x, step);
+        __syncthreads();
+        const bool f64 = MODE == kEnsF64 || (MODE == kEnsMixed && E.members[it.x].storage == ST_F64);
         if (MODE != kEnsF64 && !f64)
-          step_tile<19, S32, 32, kEnsTy, 1>(A, it.y, it.z, smem, n, d);
+          pair_tile<19, S32, 32, kEnsTy, true, GEN>(args[0], it.y, it.z, smem, n, d, tid, PairStep<GEN>(), CtaSync());
         else if (MODE == kEnsF64 || MODE == kEnsMixed)
-          step_tile<19, ST_F64, 32, kEnsTy, 1>(A, it.y, it.z, smem, n, d);
+          pair_tile<19, ST_F64, 32, kEnsTy, false, GEN>(args[0], it.y, it.z, smem, n, d, tid, PairStep<GEN>(), CtaSync());
         block_sum<NT>(n, d);
         if (tid == 0) {
           pr[w] = d;
@@ -157,26 +180,22 @@ __global__ void __launch_bounds__(kEnsThreads, MODE == kEnsF32 || MODE == kEnsF3
       } else {
         const int pack = w - E.n3;
         const int4 it = E.items[E.n3 + pack * G + grp];
-        int iters = 0;
-        for (int g = 0; g < G; ++g) iters = max(iters, E.items[E.n3 + pack * G + g].w);
         // the pack's storage: that of its first item, which is never a filler
         const bool f64 = MODE == kEnsF64 ||
                          (MODE == kEnsMixed && E.members[E.items[E.n3 + pack * G].x].storage == ST_F64);
         unsigned char* gs = smem + grp * (f64 ? ens_group_smem<G, ST_F64>() : ens_group_smem<G, S32>());
         if (it.x >= 0) {
-          const EnsMember& M = E.members[it.x];
-          StepArgs A = M.a;
-          const int c = (E.cur[it.x] + step) & 1;
-          A.pin = M.state[c];
-          A.pout = M.state[c ^ 1];
-          A.mask_in = M.mask[c];
-          A.mask_out = M.mask[c ^ 1];
+          typename GroupSyncOf<GT>::type sync;
+          if constexpr (GT != 32) sync.group = grp;
+          StepArgs& A = args[grp];
+          load_args(A, it.x, gtid, GT);
+          sync.wait();
+          if (gtid == 0) set_buffers(A, it.x, step);
+          sync.wait();
           if (MODE != kEnsF64 && !f64)
-            step_tile<9, S32, GT, 1, 1>(A, it.y, it.z, gs, n, d, gtid, iters);
+            pair_tile<9, S32, GT, 1, true, GEN>(A, it.y, it.z, gs, n, d, gtid, PairStep<GEN>(), sync);
           else if (MODE == kEnsF64 || MODE == kEnsMixed)
-            step_tile<9, ST_F64, GT, 1, 1>(A, it.y, it.z, gs, n, d, gtid, iters);
-        } else {
-          for (int r = 0; r < 1 + iters; ++r) __syncthreads();  // same barrier rounds, no work
+            pair_tile<9, ST_F64, GT, 1, false, GEN>(A, it.y, it.z, gs, n, d, gtid, PairStep<GEN>(), sync);
         }
         // per-group sums: warp shuffles, then the group's warps in shared memory
 #pragma unroll
@@ -238,18 +257,21 @@ __global__ void __launch_bounds__(kEnsThreads, MODE == kEnsF32 || MODE == kEnsF3
 template <int G, int MODE>
 static int ens_smem() {
   constexpr int S32 = ens_s32<MODE>();
-  constexpr int b32 = G * ens_group_smem<G, S32>() > TileSmem<19, S32, 32, kEnsTy, 1>::BYTES
+  constexpr int b32 = G * ens_group_smem<G, S32>() > PairSmem<19, S32, 32, kEnsTy>::BYTES
                           ? G * ens_group_smem<G, S32>()
-                          : TileSmem<19, S32, 32, kEnsTy, 1>::BYTES;
-  constexpr int b64 = G * ens_group_smem<G, ST_F64>() > TileSmem<19, ST_F64, 32, kEnsTy, 1>::BYTES
+                          : PairSmem<19, S32, 32, kEnsTy>::BYTES;
+  constexpr int b64 = G * ens_group_smem<G, ST_F64>() > PairSmem<19, ST_F64, 32, kEnsTy>::BYTES
                           ? G * ens_group_smem<G, ST_F64>()
-                          : TileSmem<19, ST_F64, 32, kEnsTy, 1>::BYTES;
+                          : PairSmem<19, ST_F64, 32, kEnsTy>::BYTES;
   return MODE == kEnsF32 || MODE == kEnsF32X ? b32 : (MODE == kEnsF64 ? b64 : (b32 > b64 ? b32 : b64));
 }
 
+// plain: no active member has links, site bytes to read or a flux field (FP32 and F32X modes).
 template <int G, int MODE>
-static const void* ens_fn() {
-  return (const void*)cg_ensemble_kernel<G, MODE>;
+static const void* ens_fn(bool plain) {
+  if constexpr (MODE == kEnsF32 || MODE == kEnsF32X)
+    if (plain) return (const void*)cg_ensemble_kernel<G, MODE, false>;
+  return (const void*)cg_ensemble_kernel<G, MODE, true>;
 }
 
 }  // namespace cgevap
@@ -278,6 +300,7 @@ struct cgevap_ens {
   unsigned long long barrier_ns = 4000000000ull;
   int skip_cta = -1, skip_step = -1;   // test hook of the grid barrier
   // plan
+  bool plain = false;    // the launch needs no general members (see ens_fn)
   int groups = 4;        // D2Q9 items per CTA
   int pc3 = 16, pc2 = 32;
   int n3 = 0, npack = 0, nitems = 0;
@@ -305,16 +328,16 @@ int efail(cgevap_ens* e, int code, const std::string& m) {
       return efail((e), CGEVAP_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(r_)); \
   } while (0)
 
-const void* kernel_for_groups(int g, int mode) {
+const void* kernel_for_groups(int g, int mode, bool plain) {
   switch (g * 4 + mode) {
-    case 2 * 4 + kEnsF32: return ens_fn<2, kEnsF32>();
-    case 4 * 4 + kEnsF32: return ens_fn<4, kEnsF32>();
-    case 2 * 4 + kEnsF64: return ens_fn<2, kEnsF64>();
-    case 4 * 4 + kEnsF64: return ens_fn<4, kEnsF64>();
-    case 2 * 4 + kEnsMixed: return ens_fn<2, kEnsMixed>();
-    case 4 * 4 + kEnsMixed: return ens_fn<4, kEnsMixed>();
-    case 2 * 4 + kEnsF32X: return ens_fn<2, kEnsF32X>();
-    case 4 * 4 + kEnsF32X: return ens_fn<4, kEnsF32X>();
+    case 2 * 4 + kEnsF32: return ens_fn<2, kEnsF32>(plain);
+    case 4 * 4 + kEnsF32: return ens_fn<4, kEnsF32>(plain);
+    case 2 * 4 + kEnsF64: return ens_fn<2, kEnsF64>(plain);
+    case 4 * 4 + kEnsF64: return ens_fn<4, kEnsF64>(plain);
+    case 2 * 4 + kEnsMixed: return ens_fn<2, kEnsMixed>(plain);
+    case 4 * 4 + kEnsMixed: return ens_fn<4, kEnsMixed>(plain);
+    case 2 * 4 + kEnsF32X: return ens_fn<2, kEnsF32X>(plain);
+    case 4 * 4 + kEnsF32X: return ens_fn<4, kEnsF32X>(plain);
     default: return nullptr;
   }
 }
@@ -441,11 +464,15 @@ int build_plan(cgevap_ens* e) {
   EN_CUDA(e, cudaMemcpyAsync(e->d_members, e->h_members.data(), e->n * sizeof(EnsMember),
                              cudaMemcpyHostToDevice, e->stream));
   // resident CTAs
-  const void* fn = kernel_for_groups(e->groups, e->mode);
   e->smem = smem_for_groups(e->groups, e->mode);
-  EN_CUDA(e, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, e->smem));
   int occ = 0, sms = 0;
-  EN_CUDA(e, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kEnsThreads, e->smem));
+  for (bool plain : {false, true}) {
+    const void* fn = kernel_for_groups(e->groups, e->mode, plain);
+    EN_CUDA(e, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, e->smem));
+    int o = 0;
+    EN_CUDA(e, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, fn, kEnsThreads, e->smem));
+    occ = plain ? std::min(occ, o) : o;
+  }
   EN_CUDA(e, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, e->device));
   if (occ < 1) return efail(e, CGEVAP_ERR_UNSUPPORTED, "ensemble kernel does not fit on an SM");
   e->grid = std::min(occ * sms, std::max(1, e->n3 + e->npack));
@@ -486,7 +513,7 @@ int launch(cgevap_ens* e, int nsteps) {
   // arrivals, generation and work counters start at zero (a launch whose barrier gave up may
   // have left arrivals counted and counters set)
   EN_CUDA(e, cudaMemsetAsync(e->d_bar, 0, 4 * sizeof(unsigned int), e->stream));
-  EN_CUDA(e, cudaLaunchKernelExC(&cfg, kernel_for_groups(e->groups, e->mode), args));
+  EN_CUDA(e, cudaLaunchKernelExC(&cfg, kernel_for_groups(e->groups, e->mode, e->plain), args));
   return CGEVAP_OK;
 }
 
@@ -631,6 +658,7 @@ int cgevap_ensemble_step(cgevap_ens* e, int nsteps) {
   for (cgevap_sim* s : e->sims)  // per-step work the persistent kernel does not do
     if (s->outlet_rho[0] > 0.0 || s->outlet_rho[1] > 0.0 || s->heat.on)
       return efail(e, CGEVAP_ERR_UNSUPPORTED, "ensemble members run neither outlets nor a heated flux");
+  bool plain = true;
   // the member table carries each member's flux, physics and solids of the moment, and the
   // buffer each state sits in; refresh both before the (graph) launch
   for (int j = 0; j < e->n; ++j) {
@@ -639,6 +667,11 @@ int cgevap_ensemble_step(cgevap_ens* e, int nsteps) {
     e->h_members[j].a.ph = v.ph;
     e->h_members[j].a.g.links = v.g.links;
     e->cur[j] = *v.cur;
+    if (e->active[j] && (v.g.links || v.ph.phi_field || v.ph.rule != 1)) plain = false;
+  }
+  if (plain != e->plain) {  // the cached graph launches the other instantiation
+    drop_graph(e);
+    e->plain = plain;
   }
   EN_CUDA(e, cudaMemcpyAsync(e->d_members, e->h_members.data(), e->n * sizeof(EnsMember),
                              cudaMemcpyHostToDevice, e->stream));

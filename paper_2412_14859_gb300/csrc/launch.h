@@ -24,12 +24,17 @@ inline int num_tile_variants(int q) { return q == 19 ? kNumTiles3D : kNumTiles2D
 // Fused step kernels (step_f64.cu, step_f32.cu, step_dev.cu): the __global__ function of a
 // (lattice, storage, tile variant), launched with `threads` threads and one StepArgs argument.
 struct KernelRef {
-  const void* fn;
+  const void* fn;     // any lattice of that kind
   int threads;
   int smem = 0;       // dynamic shared memory bytes
   int tx = 0, ty = 0; // tile shape (0: take it from tile_cfg)
   int needs_map = 0;  // 1: second kernel argument is the TMA tensor map of the input state
+  const void* plain = nullptr;  // the same step without links, site bytes read or a flux field
 };
+// The instantiation that runs step arguments a.
+inline const void* step_fn(const KernelRef& k, const StepArgs& a) {
+  return k.plain && !a.g.links && a.ph.rule == 1 && !a.ph.phi_field ? k.plain : k.fn;
+}
 KernelRef step_kernel_f64(int q, int variant);
 KernelRef step_kernel_f32(int q, int variant);
 KernelRef step_kernel_f32x(int q, int variant);  // FP32 pairs, exact colour masses (step_f32.cu)

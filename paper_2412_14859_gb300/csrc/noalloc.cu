@@ -247,7 +247,7 @@ extern "C" CGEVAP_API int cgevap_step_static_scratch(
   a.mask_in = dev_mask_in;
   a.mask_out = dev_mask_out;
   void* args[] = {&a};
-  const cudaError_t lrc = cudaLaunchKernel(k.fn, dim3((unsigned)tiles, (unsigned)nchunk),
+  const cudaError_t lrc = cudaLaunchKernel(step_fn(k, a), dim3((unsigned)tiles, (unsigned)nchunk),
                                            dim3(k.threads), args, k.smem, stream);
   if (lrc != cudaSuccess)
     return fail(CGEVAP_ERR_CUDA, std::string("static-scratch step: launch: ") + cudaGetErrorString(lrc));

@@ -1,39 +1,27 @@
 // step_f64.cu -- instantiations of the fused step for ST_F64 storage.
 #include "launch.h"
-#include "step_kernel.cuh"
+#include "pair_tile.cuh"
 
 namespace cgevap {
 
-template <int Q, int TX, int TY, int MINB, int CPT>
+template <int Q, int TX, int TY, int MINB>
 static KernelRef reg_ref() {
-  constexpr int smem = TileSmem<Q, ST_F64, TX, TY, CPT>::BYTES;
-  const void* fn = (const void*)cg_step_kernel<Q, ST_F64, TX, TY, MINB, CPT>;
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-      return {nullptr, 0};
-    attr = true;
-  }
-  KernelRef k{fn, TX * TY};
-  k.smem = smem;
-  k.tx = TX;
-  k.ty = TY * CPT;
-  return k;
+  return pair_ref<Q, ST_F64, TX, TY, MINB, false>();
 }
 
 KernelRef step_kernel_f64(int q, int variant) {
   if (q == 19) {
     switch (variant) {
-      case 0: return reg_ref<19, 16, 8, 2, 1>();
-      case 1: return reg_ref<19, 32, 8, 1, 2>();
-      case 2: return reg_ref<19, 16, 16, 1, 1>();
-      case 3: return reg_ref<19, 32, 8, 2, 1>();
-      case 4: return reg_ref<19, 32, 4, 2, 1>();
+      case 0: return reg_ref<19, 16, 8, 2>();
+      case 1: return reg_ref<19, 32, 8, 1>();
+      case 2: return reg_ref<19, 16, 16, 1>();
+      case 3: return reg_ref<19, 32, 8, 2>();
+      case 4: return reg_ref<19, 32, 4, 2>();
     }
   } else if (q == 9) {
     switch (variant) {
-      case 0: return reg_ref<9, 128, 1, 1, 1>();
-      case 1: return reg_ref<9, 64, 1, 2, 1>();
+      case 0: return reg_ref<9, 128, 1, 1>();
+      case 1: return reg_ref<9, 64, 1, 2>();
     }
   }
   return {nullptr, 0};

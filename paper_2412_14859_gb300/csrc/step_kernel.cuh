@@ -1,13 +1,14 @@
-// step_kernel.cuh -- the fused timestep: one pass over HBM per step.
+// step_kernel.cuh -- the fused timestep of the staged layouts: one pass over HBM per step.
 //
-// Work decomposition.  A CTA owns a tile of TX x TY columns of the (a, b) plane (TY = 1 for
-// D2Q9) and marches along m through a chunk of PC planes.  For every plane it
+// Work decomposition (pair_tile.cuh, for FP64 and FP32 pairs, decomposes the step the same way).
+// A CTA owns a tile of TX x TY columns of the (a, b) plane (TY = 1 for D2Q9) and marches along m
+// through a chunk of PC planes.  For every plane it
 //   (1) pulls the populations of plane m+1 (Eq. Stream, pull form, halfway bounce-back),
 //       decides the evaporation sites and applies Eq. (exchange), and writes the post-exchange
 //       phase field rho^N of the tile plus a one-cell ring into a 4-plane shared-memory ring;
 //   (2) after one __syncthreads, collides plane m (moments, Eq. cg stencil from the ring,
 //       Eq. collision/feq, Eq. perturb, Eq. recolor) from populations it pulled one iteration
-//       earlier and still holds in registers, and stores them.
+//       earlier, and stores them.
 // The ring cells around the tile (and the planes m0-1, m0+PC at the chunk ends) are pulled by
 // this CTA as well -- redundant loads that hit L2 -- so each population is read from HBM once
 // and written once per step.  Site counts and the removed mass are reduced with warp shuffles
@@ -641,7 +642,7 @@ __device__ __forceinline__ void collide_store(const StepArgs& A, int si, int nim
         rc_pop[si + dimg[j]] = fi0;
         rc_rec[si + dimg[j]] = rec;
       }
-  } else if constexpr (!Storage<S>::dev && !ExactPairs<S>::value) {
+  } else if constexpr (!Storage<S>::dev) {
     IO::store(A.pout, A.g.nstore, 0, si, f0.r, f0.b, f0, ph);
     if (GHOSTS && nimg)
       for (int j = 0; j < nimg; ++j) IO::store(A.pout, A.g.nstore, 0, si + dimg[j], f0.r, f0.b, f0, ph);
@@ -741,10 +742,6 @@ __device__ __forceinline__ void collide_store(const StepArgs& A, int si, int nim
     } else {
       IO::store(A.pout, A.g.nstore, i, si, fri, fi - fri, f0, ph);
       IO::store(A.pout, A.g.nstore, j, si, frj, fj - frj, f0, ph);
-      if constexpr (ExactPairs<S>::value) {  // what the stored moving pairs carry, exactly
-        fast_two_sum_acc(rc_out_hi, rc_out_lo, make_float2(fri, fi - fri));
-        fast_two_sum_acc(rc_out_hi, rc_out_lo, make_float2(frj, fj - frj));
-      }
       if (GHOSTS && nimg) {  // periodic ghost images: cells within two of a periodic x or y edge
         for (int k = 0; k < nimg; ++k) {
           IO::store(A.pout, A.g.nstore, i, si + dimg[k], fri, fi - fri, f0, ph);
@@ -752,20 +749,6 @@ __device__ __forceinline__ void collide_store(const StepArgs& A, int si, int nim
         }
       }
     }
-  }
-  if constexpr (ExactPairs<S>::value) {
-    // the rest pair: the exact colour masses (rr + lr, rb + lb) less the stored moving pairs
-    // (rc_out_hi - B + rc_out_lo), as for the 16-bit recolour-on-pull layout
-    rc_out_hi = sub2(rc_out_hi, sum_start(ph));  // exact
-    const float2 t = make_float2(float(rr), float(rb));
-    const float2 s2 = sub2(t, rc_out_hi);
-    const float2 e2 = make_float2(two_sum_err(t.x, -rc_out_hi.x, s2.x),
-                                  two_sum_err(t.y, -rc_out_hi.y, s2.y));
-    const float2 small = __fadd2_rn(e2, sub2(make_float2(float(lr), float(lb)), rc_out_lo));
-    const float2 r0 = __fadd2_rn(s2, small);
-    IO::store(A.pout, A.g.nstore, 0, si, r0.x, r0.y, f0, ph);
-    if (GHOSTS && nimg)
-      for (int j = 0; j < nimg; ++j) IO::store(A.pout, A.g.nstore, 0, si + dimg[j], r0.x, r0.y, f0, ph);
   }
   if constexpr (Storage<S>::rc16) {
     // the rest pair carries the exact colour masses (rr + lr, rb + lb) less what the moving
@@ -842,22 +825,9 @@ __device__ __forceinline__ int image_deltas(const Geom& g, int a, int b, int (&d
 // keeps each f_i), rho_r, rho_b and the neighbour phase field rnb are at hand: Eq.
 // (collision) to Eq. (recolor) and the store, the site byte of this step and the ledger terms.
 struct StepEpilogue {
-  // Called for each own fluid cell of plane m (storage index si) at the start of the iteration
-  // that collides plane m, before the pulls of plane m + 1: an epilogue that reads per-cell data
-  // of plane m can start fetching it here (the step itself reads nothing more).
-  template <int Q, int S>
-  __device__ __forceinline__ void prefetch(const StepArgs&, int /*si*/) const {}
-  // Called by every thread of the tile (origin a0, b0), for plane um, before the barrier that
-  // precedes the collision of plane um - 1 (and for the chunk's planes m0 - 1 and m0 before the
-  // first one): an epilogue that reads per-cell data of the neighbours stages it here.
-  template <int Q, int S>
-  __device__ __forceinline__ void stage(const StepArgs&, int /*a0*/, int /*b0*/, int /*um*/,
-                                        int /*tid*/) const {}
-  // sl, sbits, m: the cell's slot, solid-link bits and plane.  (lr, lb): the rounding errors of
-  // rr, rb (16-bit storages: rr + lr is the exact mass)
+  // (lr, lb): the rounding errors of rr, rb (16-bit storages: rr + lr is the exact mass)
   template <int Q, int S, class R>
-  __device__ __forceinline__ void cell(const StepArgs& A, int cell, const Slot& /*sl*/,
-                                       uint32_t /*sbits*/, int /*m*/, int si, int nimg,
+  __device__ __forceinline__ void cell(const StepArgs& A, int cell, int si, int nimg,
                                        const int (&dimg)[3], const R (&f)[Q], R rr, R rb,
                                        R irho, R e, uint32_t flags, const R (&rnb)[Q],
                                        int& n_sites, R& removed, R lr = R(0), R lb = R(0)) const {
@@ -902,19 +872,10 @@ struct TileSmem {
 // along m.  CPT cells per thread: thread (lx, ly) owns the columns (lx, ly + c TY), c < CPT, of a
 // TX x (TY CPT) tile, so its pulls of all CPT cells are in flight together.  smem points to
 // TileSmem<...>::BYTES bytes of shared memory.  Returns this thread's site count and removed mass.
-// tid: this thread's index within the TX*TY threads that run the tile; iters >= the number of
-// planes of the chunk: the loop runs that many barrier rounds (the extra ones idle), so several
-// tiles with different chunk lengths can share one CTA's barriers.  epi: the per-cell tail
-// (StepEpilogue for the step itself; the adjoint passes its own).
-// PF (storages that pull pairs from global memory without staging): the own cells' pulls of the
-// next plane are issued one fill ahead, into registers, so their loads are in flight during the
-// rest of that fill, the barrier and the collision of the current plane instead of being waited
-// for at once (the same values, loaded earlier; more registers live across the collision).
-template <int Q, int S, int TX, int TY, int CPT, class Epi = StepEpilogue, bool PF = false>
+template <int Q, int S, int TX, int TY, int CPT>
 __device__ __forceinline__ void step_tile(const StepArgs& A, int tile, int chunk, unsigned char* smem,
-                                          long long& n_sites, double& removed,
-                                          int tid = threadIdx.x, int iters = -1,
-                                          const Epi& epi = Epi()) {
+                                          long long& n_sites, double& removed) {
+  const int tid = threadIdx.x;
   using SM = TileSmem<Q, S, TX, TY, CPT>;
   unsigned char* ring_mem = smem;
   unsigned char* rest_mem = smem + SM::RING;
@@ -933,7 +894,6 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, int tile, int chunk
   R(*ring)[HY][HX] = reinterpret_cast<R(*)[HY][HX]>(ring_mem);
   // deviation storage: rest pairs of the tile plus a two-cell ring, planes m .. m+2
   constexpr bool DEV = Storage<S>::dev;
-  constexpr bool EXACTP = ExactPairs<S>::value;      // FP32 pairs with exact colour masses
   constexpr bool RCIN = Storage<S>::rc_in;          // reads a recolour-on-pull layout
   constexpr bool RC16IN = RCIN && Storage<S>::rc16;  // ... the 16-bit one
   constexpr bool STAGE = DEV || RCIN;    // pulls read per-source data staged in shared memory
@@ -1102,28 +1062,6 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, int tile, int chunk
 
   // Pull plane um for the own cells and the ring cell; write rho^N to the ring; the own cells'
   // post-exchange populations are returned in g.
-  // PF: the own cells' pulls issued one fill ahead (storages whose pulls need nothing staged; the
-  // 16-bit ones are bound by their instruction count, not by load latency, and gain nothing)
-  static_assert(!(PF && STAGE), "pulls issued ahead only for storages without staged sources");
-  V2<R> pf[CPT][Q];   // PF: the own cells' pulled populations of the next plane to fill
-  uint32_t pfbits[CPT];
-  bool pfok[CPT];
-  (void)pf;
-  auto issue = [&](int um) {  // PF: issue the own cells' pulls of plane um
-    if constexpr (PF) {
-      const Plane p = make_plane(G, um);
-      const PlaneOffsets po = plane_offsets(G, p.m);
-#pragma unroll
-      for (int c = 0; c < CPT; ++c) {
-        const int cl = (p.m * G.nb + me[c].b) * G.na + me[c].a;
-        uint32_t bits = 0;
-        pfok[c] = solid_bits<L>(G, me[c], p, cl, bits);
-        pfbits[c] = bits;
-        if (pfok[c]) pull_cell<Q, S>(A, me[c], sidx(G, me[c].a, me[c].b, p.m), po, bits, pf[c]);
-      }
-    }
-  };
-  (void)issue;
   auto fill_plane = [&](int um, CellScalars(&out)[CPT], V2<R>(&g)[CPT][Q]) {
     const Plane p = make_plane(G, um);
     const PlaneOffsets po = plane_offsets(G, p.m);
@@ -1171,13 +1109,6 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, int tile, int chunk
 #pragma unroll
     for (int c = 0; c < CPT; ++c) {  // issue every load of every own cell first
       cells[c] = (p.m * G.nb + me[c].b) * G.na + me[c].a;
-      if constexpr (PF) {  // issued one fill ahead
-        out[c].ok = pfok[c];
-        out[c].bits = pfbits[c];
-#pragma unroll
-        for (int i = 0; i < Q; ++i) g[c][i] = pf[c][i];
-        continue;
-      }
       uint32_t bits = 0;
       out[c].ok = solid_bits<L>(G, me[c], p, cells[c], bits);
       out[c].bits = bits;
@@ -1201,7 +1132,6 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, int tile, int chunk
           pull_cell<Q, S>(A, me[c], sidx(G, me[c].a, me[c].b, p.m), po, bits, g[c]);
       }
     }
-    issue(um + 1);  // PF: the next fill's own pulls, in flight from here
 #pragma unroll
     for (int c = 0; c < CPT; ++c) {
       R rn = R(0);
@@ -1214,27 +1144,6 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, int tile, int chunk
             out[c].lr = __fadd_rn(out[c].lr, two_sum_err(sr, -out[c].e, out[c].rr));
             out[c].lb = __fadd_rn(out[c].lb, two_sum_err(sb, out[c].e, out[c].rb));
           }
-        } else if constexpr (EXACTP) {
-          // the plain sums of the FP32 pairs (those the ring cells form, so rho^N of a cell is
-          // the same in every tile that holds it) and the colour totals without rounding error
-          // (from B); what the exact totals exceed the plain ones by, and the exchange's own
-          // rounding (TwoSum), go to (lr, lb)
-          float2 plain = make_float2(0.0f, 0.0f);
-          float2 acc = sum_start(A.ph), lo = make_float2(0.0f, 0.0f);
-#pragma unroll
-          for (int i = 0; i < Q; ++i) {
-            const float2 v = make_float2(g[c][i].r, g[c][i].b);
-            plain = __fadd2_rn(plain, v);
-            fast_two_sum_acc(acc, lo, v);
-          }
-          // (acc - B) and plain are both within a few ulps of B of the total: exact difference
-          lo = __fadd2_rn(sub2(sub2(acc, sum_start(A.ph)), plain), lo);
-          rn = exchange_from_sums<S>(A, cells[c], plain.x, plain.y, out[c].rr, out[c].rb,
-                                     out[c].e, out[c].flags, out[c].irho);
-          out[c].lr = __fadd_rn(lo.x, two_sum_err(plain.x, -out[c].e, out[c].rr));
-          out[c].lb = __fadd_rn(lo.y, two_sum_err(plain.y, out[c].e, out[c].rb));
-          g[c][0].r -= out[c].e;
-          g[c][0].b += out[c].e;
         } else
           rn = site_exchange<Q, S>(A, cells[c], g[c], out[c].rr, out[c].rb, out[c].e,
                                    out[c].flags, out[c].irho);
@@ -1249,9 +1158,6 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, int tile, int chunk
       stage_rest(um + 2);
   };
 
-  epi.template stage<Q, S>(A, a0, b0, m0 - 1, tid);
-  epi.template stage<Q, S>(A, a0, b0, m0, tid);
-  issue(m0 - 1);  // PF: the first fill's own pulls
   stage_rest(m0 - 2);
   stage_rest(m0 - 1);
   stage_rest(m0);
@@ -1273,16 +1179,7 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, int tile, int chunk
   }
   if (STAGE) __syncthreads();  // the first fill below restages a slot the pulls above read
 
-  const int m_end = iters < 0 ? m1 : m0 + iters;
-  for (int m = m0; m < m_end; ++m) {
-    if (m >= m1) {  // idle barrier rounds of a shorter chunk sharing the CTA
-      __syncthreads();
-      continue;
-    }
-    epi.template stage<Q, S>(A, a0, b0, m + 1, tid);
-#pragma unroll
-    for (int c = 0; c < CPT; ++c)
-      if (active[c] && cur[c].ok) epi.template prefetch<Q, S>(A, sidx(G, me[c].a, me[c].b, m));
+  for (int m = m0; m < m1; ++m) {
     V2<R> g[CPT][Q];
     fill_plane(m + 1, nxt, g);
     __syncthreads();
@@ -1314,13 +1211,11 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, int tile, int chunk
         }
       }
       const int cell = (m * G.nb + me[c].b) * G.na + me[c].a;
-      if constexpr (DEV || RC16IN || EXACTP)
-        epi.template cell<Q, S>(A, cell, me[c], cur[c].bits, m, sidx(G, me[c].a, me[c].b, m),
-                                nimg[c], dimg[c], own, cur[c].rr, cur[c].rb, cur[c].irho,
+      if constexpr (DEV || RC16IN)
+        StepEpilogue().template cell<Q, S>(A, cell, sidx(G, me[c].a, me[c].b, m), nimg[c], dimg[c], own, cur[c].rr, cur[c].rb, cur[c].irho,
                                 cur[c].e, cur[c].flags, rnb, nloc, rem, cur[c].lr, cur[c].lb);
       else
-        epi.template cell<Q, S>(A, cell, me[c], cur[c].bits, m, sidx(G, me[c].a, me[c].b, m),
-                                nimg[c], dimg[c], own, cur[c].rr, cur[c].rb, cur[c].irho,
+        StepEpilogue().template cell<Q, S>(A, cell, sidx(G, me[c].a, me[c].b, m), nimg[c], dimg[c], own, cur[c].rr, cur[c].rb, cur[c].irho,
                                 cur[c].e, cur[c].flags, rnb, nloc, rem);
     }
 #pragma unroll
@@ -1400,12 +1295,12 @@ __device__ __forceinline__ void ledger_fold(const Reduce& red, long long n, doub
   }
 }
 
-template <int Q, int S, int TX, int TY, int MINB, int CPT, bool PF = false>
+template <int Q, int S, int TX, int TY, int MINB, int CPT>
 __global__ void __launch_bounds__(TX* TY, MINB) cg_step_kernel(const __grid_constant__ StepArgs A) {
   extern __shared__ __align__(16) unsigned char dyn_smem[];
   long long n = 0;
   double d = 0.0;
-  step_tile<Q, S, TX, TY, CPT, StepEpilogue, PF>(A, blockIdx.x, blockIdx.y, dyn_smem, n, d);
+  step_tile<Q, S, TX, TY, CPT>(A, blockIdx.x, blockIdx.y, dyn_smem, n, d);
   block_sum<TX * TY>(n, d);
   ledger_fold(A.red, n, d);
 }
