@@ -170,18 +170,6 @@ __device__ __forceinline__ void collide_adjoint(const Physics& ph, const CellMom
   }
 }
 
-// Asynchronous copy of `bytes` (8 or 16) from global to shared memory, and its completion for
-// the issuing thread (cp.async; the copies land while the thread goes on).
-template <int BYTES>
-__device__ __forceinline__ void async_copy(void* smem_dst, const void* gsrc) {
-  static_assert(BYTES == 8 || BYTES == 16, "cp.async copies 4, 8 or 16 bytes");
-  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(gsrc), "n"(BYTES)
-               : "memory");
-}
-__device__ __forceinline__ void async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
 // Kernel A's per-cell tail (replaces StepEpilogue in step_tile).  It reads lambda^{n+1} and
 // writes the transpose of the pull of step n directly:
 //   lambda^n_j(y) = lg_j(y + c_j) + ab(y + c_j), or lg_{opp j}(y) + ab(y) where y + c_j is solid

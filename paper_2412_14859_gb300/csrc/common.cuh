@@ -348,7 +348,7 @@ struct PopIO<S, Q, true> {
                                                       float r, float b, V2<float> f0,
                                                       const Physics& ph) {
     P* d = reinterpret_cast<P*>(reinterpret_cast<char*>(base) + dev_block_offset(nstore)) +
-           (size_t)(i - 1) * nstore + si;
+           ((i - 1) * nstore + si);
     const float2 dev = __fmul2_rn(
         __ffma2_rn(make_float2(-f0.r, -f0.b), make_float2(ph.kap_r[i], ph.kap_b[i]), make_float2(r, b)),
         make_float2(ph.scale, ph.scale));
@@ -369,7 +369,7 @@ struct PopIO<S, Q, true> {
     if (i == 0) return {f0.x, f0.y};
     const P* d = reinterpret_cast<const P*>(reinterpret_cast<const char*>(base) +
                                             dev_block_offset(nstore)) +
-                 (size_t)(dir - 1) * nstore + si;
+                 ((dir - 1) * nstore + si);
     const float2 v = Storage<S>::unpack(__ldg(d));
     const float2 r = __ffma2_rn(f0, make_float2(ph.kap_r[i], ph.kap_b[i]),
                                 __fmul2_rn(v, make_float2(ph.inv_scale, ph.inv_scale)));
@@ -382,7 +382,7 @@ struct PopIO<S, Q, true> {
       return;
     }
     P* d = reinterpret_cast<P*>(reinterpret_cast<char*>(base) + dev_block_offset(nstore)) +
-           (size_t)(i - 1) * nstore + si;
+           ((i - 1) * nstore + si);
     // (f - f0 kappa) scale for both components in packed FP32
     const float2 dev = __fmul2_rn(
         __ffma2_rn(make_float2(-f0.r, -f0.b), make_float2(ph.kap_r[i], ph.kap_b[i]), make_float2(r, b)),

@@ -117,6 +117,18 @@ __device__ __forceinline__ typename Storage<S>::real flux_at(const Physics& ph, 
   return (R)__ldg(reinterpret_cast<const R*>(ph.phi_field) + cell) * PHYS(R, ph, inv_sbar);
 }
 
+// Asynchronous copy of `bytes` (4, 8 or 16) from global to shared memory, and its completion for
+// the issuing thread (cp.async; the copies land while the thread goes on).
+template <int BYTES>
+__device__ __forceinline__ void async_copy(void* smem_dst, const void* gsrc) {
+  static_assert(BYTES == 4 || BYTES == 8 || BYTES == 16, "cp.async copies 4, 8 or 16 bytes");
+  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(gsrc), "n"(BYTES)
+               : "memory");
+}
+__device__ __forceinline__ void async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 template <class R>
 __device__ __forceinline__ R recip(R x);
 template <>
@@ -300,7 +312,7 @@ __device__ __forceinline__ void pull_cell_dev(const StepArgs& A, const Slot& sl,
       const int src = si + (L::ca(i) > 0 ? sl.dxm : (L::ca(i) < 0 ? sl.dxp : 0)) +
                       (L::cb(i) > 0 ? sl.dym : (L::cb(i) < 0 ? sl.dyp : 0)) +
                       (L::cm(i) > 0 ? po.dm_lo : (L::cm(i) < 0 ? po.dm_hi : 0));
-      const P v = __ldg(dev + (i - 1) * ns + src);
+      const P v = __ldg(dev + ((i - 1) * ns + src));
       raw[i] = *reinterpret_cast<const uint32_t*>(&v);
     }
 #pragma unroll
@@ -323,7 +335,7 @@ __device__ __forceinline__ void pull_cell_dev(const StepArgs& A, const Slot& sl,
       const bool bounce = (sbits >> i) & 1u;
       src = bounce ? si : src;
       const int dir = bounce ? opp(i) : i;
-      const P v = __ldg(dev + (size_t)(dir - 1) * ns + src);
+      const P v = __ldg(dev + ((dir - 1) * ns + src));
       raw[i] = *reinterpret_cast<const uint32_t*>(&v);
     }
 #pragma unroll
@@ -370,7 +382,7 @@ __device__ __forceinline__ void pull_cell_rc(const StepArgs& A, const Slot& sl, 
       const int src = si + (L::ca(i) > 0 ? sl.dxm : (L::ca(i) < 0 ? sl.dxp : 0)) +
                       (L::cb(i) > 0 ? sl.dym : (L::cb(i) < 0 ? sl.dyp : 0)) +
                       (L::cm(i) > 0 ? po.dm_lo : (L::cm(i) < 0 ? po.dm_hi : 0));
-      fv[i] = __ldg(pop + i * ns + src);
+      fv[i] = __ldg(pop + (i * ns + src));
     }
   } else {
 #pragma unroll
@@ -381,7 +393,7 @@ __device__ __forceinline__ void pull_cell_rc(const StepArgs& A, const Slot& sl, 
       const bool bounce = (sbits >> i) & 1u;
       src = bounce ? si : src;
       const int dir = bounce ? opp(i) : i;
-      fv[i] = __ldg(pop + (size_t)dir * ns + src);
+      fv[i] = __ldg(pop + (dir * ns + src));
     }
   }
   const float4 r0 = recbox(ps[1], ey, ex);
@@ -438,7 +450,7 @@ __device__ __forceinline__ void rc16_load(const StepArgs& A, const Slot& sl, int
       const int src = si + (L::ca(i) > 0 ? sl.dxm : (L::ca(i) < 0 ? sl.dxp : 0)) +
                       (L::cb(i) > 0 ? sl.dym : (L::cb(i) < 0 ? sl.dyp : 0)) +
                       (L::cm(i) > 0 ? po.dm_lo : (L::cm(i) < 0 ? po.dm_hi : 0));
-      raw[i] = __ldg(dev + (i - 1) * ns + src);
+      raw[i] = __ldg(dev + ((i - 1) * ns + src));
     }
   } else {
 #pragma unroll
@@ -449,7 +461,7 @@ __device__ __forceinline__ void rc16_load(const StepArgs& A, const Slot& sl, int
       const bool bounce = (sbits >> i) & 1u;
       src = bounce ? si : src;
       const int dir = bounce ? opp(i) : i;
-      raw[i] = __ldg(dev + (size_t)(dir - 1) * ns + src);
+      raw[i] = __ldg(dev + ((dir - 1) * ns + src));
     }
   }
   r0 = __ldg(reinterpret_cast<const float2*>(base) + si);
@@ -704,8 +716,8 @@ __device__ __forceinline__ void collide_store(const StepArgs& A, int si, int nim
       const float ri = float(rc16_ratio<L>(i)) * rc16_rf;  // exact (r_i is a power of two)
       const P hi = H::pack((fi - ri) * ph.scale);
       const P hj = H::pack((fj - ri) * ph.scale);
-      dev[(size_t)(i - 1) * A.g.nstore + si] = hi;
-      dev[(size_t)(j - 1) * A.g.nstore + si] = hj;
+      dev[(i - 1) * A.g.nstore + si] = hi;  // element indices in 32 bits: Q nstore < 2^31
+      dev[(j - 1) * A.g.nstore + si] = hj;
       const float di = fmaf(H::unpack(hi), ph.inv_scale, ri);
       const float dj = fmaf(H::unpack(hj), ph.inv_scale, ri);
       const float fr_i = rc_red<L>(i, rc16_rec.x, di, rc_cv<L>(i, rc16_rec));
@@ -713,7 +725,7 @@ __device__ __forceinline__ void collide_store(const StepArgs& A, int si, int nim
       fast_two_sum_acc(rc_out_hi, rc_out_lo, make_float2(fr_i, di - fr_i));
       fast_two_sum_acc(rc_out_hi, rc_out_lo, make_float2(fr_j, dj - fr_j));
     } else if constexpr (Storage<S>::rc) {
-      const size_t ns = (size_t)A.g.nstore;
+      const int ns = A.g.nstore;
       rc_pop[i * ns + si] = fi;
       rc_pop[j * ns + si] = fj;
       if (GHOSTS && nimg)
@@ -974,68 +986,37 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, int tile, int chunk
   float4(*rec_ring)[RY][RX] = reinterpret_cast<float4(*)[RY][RX]>(rest_mem);
   float(*ref_ring)[RY][RX] = reinterpret_cast<float(*)[RY][RX]>(rest_mem + RS * RY * RX * 16);
   (void)ref_ring;
-  auto stage_rest = [&](int uq) {  // rest pairs / records of plane uq (unwrapped) into its slot
-    if (!STAGE) return;
-    const Plane q = make_plane(G, uq);
-    const int sl = rest_slot(uq);
-    if constexpr (RC16IN) {
-      const Rc16Layout lay = rc16_layout(Q, G.nstore);
-      const char* b = reinterpret_cast<const char*>(A.pin);
-      const float4* rec = reinterpret_cast<const float4*>(b + lay.rec);
-      const float* ref = reinterpret_cast<const float*>(b + lay.ref);
+  // Starts the copies of the rest pairs / records of plane uq (unwrapped) into its slot: asynchronous,
+  // issued at the start of a fill and waited for before the barrier that ends it, so their latency
+  // lies under the fill's pulls and no register holds them (192^3, us a step, with the 32-bit
+  // element indices: F16RC 567 -> 526, F32RC 483 -> 451; F16DEV, which already loaded early into
+  // registers, 517 -> 518, 128^3 180 -> 176).
+  auto stage_rest = [&](int uq) {
+    if constexpr (STAGE) {
+      const Plane q = make_plane(G, uq);
+      if (!q.ok) return;
+      const int sl = rest_slot(uq);
+      const char* const base = reinterpret_cast<const char*>(A.pin);
 #pragma unroll
       for (int k = 0; k < RPT; ++k) {
         const int e = tid + k * NT;
-        if (e < RN && q.ok && rest_off[k] >= 0) {
-          rec_ring[sl][e / RX][e % RX] = __ldg(rec + q.m * plane_stride + rest_off[k]);
-          ref_ring[sl][e / RX][e % RX] = __ldg(ref + q.m * plane_stride + rest_off[k]);
+        if (e >= RN || rest_off[k] < 0) continue;
+        const int at = q.m * plane_stride + rest_off[k], to = sl * RN + e;
+        if constexpr (RC16IN) {
+          const Rc16Layout lay = rc16_layout(Q, G.nstore);
+          async_copy<16>(reinterpret_cast<float4*>(rest_mem) + to, reinterpret_cast<const float4*>(base + lay.rec) + at);
+          async_copy<4>(&ref_ring[0][0][0] + to, reinterpret_cast<const float*>(base + lay.ref) + at);
+        } else if constexpr (RCIN) {
+          async_copy<16>(reinterpret_cast<float4*>(rest_mem) + to,
+                         reinterpret_cast<const float4*>(base + rc_record_offset(Q, G.nstore)) + at);
+        } else {
+          async_copy<8>(reinterpret_cast<float2*>(rest_mem) + to, reinterpret_cast<const float2*>(base) + at);
         }
       }
-    } else if constexpr (RCIN) {
-      const float4* rec = reinterpret_cast<const float4*>(reinterpret_cast<const char*>(A.pin) +
-                                                          rc_record_offset(Q, G.nstore));
-#pragma unroll
-      for (int k = 0; k < RPT; ++k) {
-        const int e = tid + k * NT;
-        if (e < RN && q.ok && rest_off[k] >= 0)
-          rec_ring[sl][e / RX][e % RX] = __ldg(rec + q.m * plane_stride + rest_off[k]);
-      }
-    } else {
-      const float2* rest = reinterpret_cast<const float2*>(A.pin);
-#pragma unroll
-      for (int k = 0; k < RPT; ++k) {
-        const int e = tid + k * NT;
-        if (e < RN && q.ok && rest_off[k] >= 0)
-          rest_ring[sl][e / RX][e % RX] = __ldg(rest + q.m * plane_stride + rest_off[k]);
-      }
     }
   };
-  // the same staging split in two: the loads of plane uq into registers (issued before the
-  // pulls of a plane, so their latency overlaps them) and their stores into its slot (after)
-  using BoxT = typename std::conditional<RCIN, float4, float2>::type;
-  auto stage_load = [&](int uq, BoxT (&v)[RPT]) {
-    if constexpr (STAGE) {
-      const Plane q = make_plane(G, uq);
-      const BoxT* src = reinterpret_cast<const BoxT*>(reinterpret_cast<const char*>(A.pin) +
-                                                      (RCIN ? rc_record_offset(Q, G.nstore) : 0));
-#pragma unroll
-      for (int k = 0; k < RPT; ++k) {
-        const int e = tid + k * NT;
-        if (e < RN && q.ok && rest_off[k] >= 0) v[k] = __ldg(src + q.m * plane_stride + rest_off[k]);
-      }
-    }
-  };
-  auto stage_store = [&](int uq, const BoxT (&v)[RPT]) {
-    if constexpr (STAGE) {
-      const Plane q = make_plane(G, uq);
-      BoxT(*ring_t)[RY][RX] = reinterpret_cast<BoxT(*)[RY][RX]>(rest_mem);
-      const int sl = rest_slot(uq);
-#pragma unroll
-      for (int k = 0; k < RPT; ++k) {
-        const int e = tid + k * NT;
-        if (e < RN && q.ok && rest_off[k] >= 0) ring_t[sl][e / RX][e % RX] = v[k];
-      }
-    }
+  auto staged = [&]() {  // before the barrier that publishes them
+    if constexpr (STAGE) async_wait_all();
   };
   auto restbox = [&](int slot, int y, int x) -> float2 { return rest_ring[slot][y][x]; };
   auto recbox = [&](int slot, int y, int x) -> float4 { return rec_ring[slot][y][x]; };
@@ -1067,13 +1048,14 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, int tile, int chunk
     const PlaneOffsets po = plane_offsets(G, p.m);
     const int slot = (um - m0 + 1) & 3;
     int ps[3] = {0, 0, 0};
-    BoxT staged[RPT];
+    // plane um + 2 into the slot of plane um - 2, which the pulls of plane um - 1 read before the
+    // last barrier; the pulls of plane um + 1 read it after the next one
+    stage_rest(um + 2);
     if (STAGE) {  // the pulls of plane um read the staged data of planes um-1 .. um+1, staged
                   // before the barrier that ended the previous plane
       ps[0] = rest_slot(um + 1);
       ps[1] = rest_slot(um);
       ps[2] = rest_slot(um - 1);
-      if constexpr (DEV) stage_load(um + 2, staged);  // registers to spare: load early
     }
     if (has_halo) {
       const int cell = (p.m * G.nb + hs.b) * G.na + hs.a;
@@ -1150,23 +1132,19 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, int tile, int chunk
       }
       ring[slot][ly0 + c * TY + OB][lx + 1] = rn;
     }
-    // plane um + 2 into the slot of plane um - 2, which the pulls of plane um - 1 read before
-    // the last barrier; the pulls of plane um + 1 read it after the next one
-    if constexpr (DEV)
-      stage_store(um + 2, staged);
-    else
-      stage_rest(um + 2);
   };
 
   stage_rest(m0 - 2);
   stage_rest(m0 - 1);
   stage_rest(m0);
+  staged();
   if (STAGE) __syncthreads();
   {
     CellScalars t[CPT];
     V2<R> g[CPT][Q];
     fill_plane(m0 - 1, t, g);
   }
+  staged();
   __syncthreads();  // the next fill restages a rest slot the pulls above may still read
   {
     V2<R> g[CPT][Q];
@@ -1177,11 +1155,13 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, int tile, int chunk
       for (int i = 0; i < Q; ++i)
         parked[(c * Q + i) * NT + tid] = STAGE ? g[c][i].r : g[c][i].r + g[c][i].b;
   }
+  staged();
   if (STAGE) __syncthreads();  // the first fill below restages a slot the pulls above read
 
   for (int m = m0; m < m1; ++m) {
     V2<R> g[CPT][Q];
     fill_plane(m + 1, nxt, g);
+    staged();
     __syncthreads();
 #pragma unroll
     for (int c = 0; c < CPT; ++c) {
