@@ -26,6 +26,12 @@
 #include "launch.h"
 #include "pair_tile.cuh"
 
+#ifndef ADJ_T
+#define ADJ_T 384
+#endif
+#ifndef ADJ_PF
+#define ADJ_PF true
+#endif
 namespace cgevap {
 
 // Minority fraction product w_r w_b below which the adjoint holds the recoloring direction fixed.
@@ -38,139 +44,209 @@ __device__ __forceinline__ int pull_source(int4 to, int lo, int hi, int si, int 
          (L::cb(i) > 0 ? to.z : (L::cb(i) < 0 ? to.w : 0)) + (L::cm(i) > 0 ? lo : (L::cm(i) < 0 ? hi : 0));
 }
 
-// (1) for one cell: from its moments c, F and the colour-blind sums f of its post-exchange
-// populations, recompute the per-direction terms of collide_pairs and run them backwards.
-// lam_at(i): lambda^{n+1} of direction i (loaded where it is used); out: lg_out(i, v) takes
-// lg_i = dL/dg_i through this cell's own collision, lF = dL/dF.
+// (1) for one cell: from its moments c0, F and the colour-blind sums f of its post-exchange
+// populations, the terms of collide_pairs run backwards.  lam_at(i): lambda^{n+1} of direction i
+// (read where it is used); out: lg_out(i, v) takes lg_i = dL/dg_i through this cell's own
+// collision, lF = dL/dF.
+//
+// With d_i = lambda^r_i - lambda^b_i and q_i = w_r d_i + lambda^b_i (dL/d of the colour-blind
+// output), the derivative with respect to every per-cell quantity is a polynomial in c_i.u and
+// c_i.e (e = F/|F|) summed over directions, so per speed class s it needs only
+//   scalars  D0 = sum d, Q0 = sum q, DU = sum d (c.u)^2, DN = sum d (c.e)^2,
+//   vectors  DV = sum d c, QV = sum q c, UV = sum q (c.u) c, PV = sum q (c.e) c,
+// plus sum d f and sum q f; opposite directions enter as sums and differences.  Kernel A is bound
+// by its instruction count, and this takes about 16 operations a direction where running each
+// direction's own chain backwards took about 45: FP32, 1.57 M cells under ncu, 99.4 M warp
+// instructions and 228 us before, 84.9 M and 177 us with it and with the pulls a plane ahead
+// (72.1 -> 69.3 ms a fit iteration of 32 steps on the full cap for the latter); FP64 fit on the
+// reduced cap 15.6 -> 12.6 ms.  At 128 registers (four CTAs per SM) it spills: 87 ms.
+//
+// Where w_r w_b < kBulkTrace (bulk: one colour is a trace) the recoloring direction e is held
+// fixed: that term is homogeneous of degree 1 in the trace, so its derivative with respect to F
+// stays O(beta w_r / |F|) however small the trace, and the linearised trace dynamics grows
+// without bound while the traces themselves stay negligible.
 template <int Q, class R, class LamAt, class LgOut>
 __device__ __forceinline__ void collide_adjoint(const Physics& ph, const CellMoments<R>& c0, const R (&f)[Q],
                                                 R irho, R Fa, R Fb, R Fm, const LamAt& lam_at,
                                                 const LgOut& lg_out, R (&lF)[3]) {
   using L = Lattice<Q>;
-  const R rho = c0.rho, wr = c0.wr, wb = c0.wb, ua = c0.ua, ub = c0.ub, um = c0.um;
-  const R uu15 = c0.uu15, itau = c0.itau, abar = c0.abar;
+  const R rho = c0.rho, wr = c0.wr, wb = c0.wb, itau = c0.itau, uu15 = c0.uu15;
+  const R u[3] = {c0.ua, c0.ub, c0.um};
   const R ir = PHYS(R, ph, inv_tau_r), ib = PHYS(R, ph, inv_tau_b);
   R F2 = fma(Fa, Fa, Fm * Fm);
   if (L::D3) F2 = fma(Fb, Fb, F2);
   R Fn = R(0), iFn = R(0);
   if (F2 > R(0)) norm_of(F2, Fn, iFn);
+  const R e[3] = {Fa * iFn, Fb * iFn, Fm * iFn};
+  // sums over the directions of speed classes 1 and 2 (index 0: the rest direction)
+  R D0[3], Q0[3], DU[3], DN[3], DV[3][3], QV[3][3], UV[3][3], PV[3][3], q[Q];
+#pragma unroll
+  for (int s = 0; s < 3; ++s) {
+    D0[s] = Q0[s] = DU[s] = DN[s] = R(0);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) DV[s][k] = QV[s][k] = UV[s][k] = PV[s][k] = R(0);
+  }
+  R Sdf, Sqf;
+  {
+    const V2<R> l = lam_at(0);
+    D0[0] = l.r - l.b;
+    q[0] = Q0[0] = fma(wr, D0[0], l.b);
+    Sdf = D0[0] * f[0];
+    Sqf = q[0] * f[0];
+  }
+#pragma unroll
+  for (int i = 1; i < Q; i += 2) {
+    const int j = i + 1, s = L::speed2(i);
+    const V2<R> li = lam_at(i), lj = lam_at(j);
+    const R di = li.r - li.b, dj = lj.r - lj.b;
+    q[i] = fma(wr, di, li.b);
+    q[j] = fma(wr, dj, lj.b);
+    Sdf = fma(dj, f[j], fma(di, f[i], Sdf));
+    Sqf = fma(q[j], f[j], fma(q[i], f[i], Sqf));
+    const R qs = q[i] + q[j], qd = q[i] - q[j], ds = di + dj, dd = di - dj;
+    R cu = R(0), ce = R(0);
+    bool any = false;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int c = axis_comp<L>(i, k);
+      if (!c) continue;
+      cu = any ? (c > 0 ? cu + u[k] : cu - u[k]) : (c > 0 ? u[k] : -u[k]);
+      ce = any ? (c > 0 ? ce + e[k] : ce - e[k]) : (c > 0 ? e[k] : -e[k]);
+      any = true;
+    }
+    Q0[s] += qs;
+    D0[s] += ds;
+    DU[s] = fma(ds * cu, cu, DU[s]);
+    DN[s] = fma(ds * ce, ce, DN[s]);
+    const R qu = qs * cu, qe = qs * ce;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int c = axis_comp<L>(i, k);
+      if (!c) continue;
+      DV[s][k] = c > 0 ? DV[s][k] + dd : DV[s][k] - dd;
+      QV[s][k] = c > 0 ? QV[s][k] + qd : QV[s][k] - qd;
+      UV[s][k] = c > 0 ? UV[s][k] + qu : UV[s][k] - qu;
+      PV[s][k] = c > 0 ? PV[s][k] + qe : PV[s][k] - qe;
+    }
+  }
   const R amp = PHYS(R, ph, amp), beta = PHYS(R, ph, beta);
-  const R pamp = amp * itau;
-  const R rcol = beta * wr * wb;
-  R restc[3], rwc[3], nrm[3], As[3], Bs[3], Ws[3], Cs[3];
+  const R pamp = amp * itau, rcol = beta * wr * wb;
+  const R rdir = wr * wb < R(kBulkTrace) ? R(0) : rcol;  // bulk: e fixed
+  R A_rcol = R(0), A_rho = R(0), A_abar = R(0), A_uu15 = R(0), Sqeq = R(0), Sdeq = R(0);
+  R Spert_q = R(0), Spert_d = R(0), Sn = R(0), Sg = R(0);
+  R Au[3] = {R(0), R(0), R(0)}, P[3] = {R(0), R(0), R(0)}, G[3] = {R(0), R(0), R(0)};
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const int i = c == 0 ? 0 : (c == 1 ? 1 : L::Q - 1);
-    As[c] = R(L::A(i));
-    Bs[c] = R(L::B(i));
-    Ws[c] = R(L::W(i));
-    Cs[c] = R(L::C(i));
-    nrm[c] = R(inv_norm<L>(i));
-    restc[c] = rho * (As[c] + Bs[c] * abar);
-    rwc[c] = rho * Ws[c];
-  }
-
-  // Backwards through recolor -> perturb -> collision -> feq, direction by direction.  The
-  // F-dependence is carried by |F| and the unit vector e = F/|F| (nc_i = e.c_i), both bounded:
-  //   perturbation  pamp (W_s |F| nc_i^2 - C_s |F|)   -> d/dF = pamp (2 W_s nc_i c_i - (W_s nc_i^2 + C_s) e)
-  //   recoloring    rcol nrm_s restc_s nc_i          -> d/dF = rcol nrm_s restc_s (c_i - nc_i e) / |F|
-  // so 1/|F| enters once (as in the step itself); far from an interface |F| can be tiny.
-  // Where w_r w_b < kBulkTrace (bulk: one colour is a trace) the recoloring direction e is held
-  // fixed: that term is homogeneous of degree 1 in the trace, so its derivative with respect to F
-  // stays O(beta w_r / |F|) however small the trace, and the linearised trace dynamics grows
-  // without bound while the traces themselves stay negligible.
-  R A_wr = R(0), A_itau = R(0), A_uu15 = R(0), A_pamp = R(0), A_rcol = R(0);
-  R A_rwc[3] = {R(0), R(0), R(0)}, A_restc[3] = {R(0), R(0), R(0)};
-  R Aua = R(0), Aub = R(0), Aum = R(0);
-  R Pa = R(0), Pb = R(0), Pm = R(0);  // sum_i 2 pamp W_s q_i nc_i c_i
-  R Ga = R(0), Gb = R(0), Gm = R(0);  // sum_i g_i c_i, g_i = d_i rcol nrm_s restc_s
-  R Sn = R(0), Sg = R(0);             // sum_i q_i (W_s nc_i^2 + C_s), sum_i g_i nc_i
-  const bool bulk = wr * wb < R(kBulkTrace);
-  R Af[Q];
+  for (int s = 0; s < 3; ++s) {
+    const int i = s == 0 ? 0 : (s == 1 ? 1 : L::Q - 1);  // a direction of speed class s
+    const R W = R(L::W(i)), C = R(L::C(i)), nrm = R(inv_norm<L>(i));
+    const R rest1 = fma(R(L::B(i)), c0.abar, R(L::A(i)));  // f_i^eq(rho, 0) / rho
+    const R restc = rho * rest1, rw = rho * W;
+    R qpoly = -uu15 * Q0[s], dpoly = -uu15 * D0[s], A_rest = itau * Q0[s];
+    if (s > 0) {
+      R uUV = R(0), uQV = R(0), uDV = R(0), eDV = R(0), ePV = R(0);
 #pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    const int c = L::speed2(i);
-    R cu = R(0), pc = R(0);
-    if (L::ca(i) > 0) { cu += ua; pc += Fa; }
-    if (L::ca(i) < 0) { cu -= ua; pc -= Fa; }
-    if (L::cb(i) > 0) { cu += ub; pc += Fb; }
-    if (L::cb(i) < 0) { cu -= ub; pc -= Fb; }
-    if (L::cm(i) > 0) { cu += um; pc += Fm; }
-    if (L::cm(i) < 0) { cu -= um; pc -= Fm; }
-    const R nc = pc * iFn;  // e.c_i (0 where F = 0)
-    const R poly = cu * (R(4.5) * cu + R(3)) - uu15;
-    const R feq = rwc[c] * poly + restc[c];
-    const R pert = Ws[c] * Fn * nc * nc - Cs[c] * Fn;  // perturbation shape, Eq. (perturb)
-    const R fi = f[i] + itau * (feq - f[i]) + pamp * pert;  // post-perturbation
-    // Eq. (recolor): f^{r*} = wr fi + rcol nrm restc nc, f^{b*} = fi - f^{r*}
-    const V2<R> li = lam_at(i);
-    const R d = li.r - li.b;
-    const R q = wr * d + li.b;  // dL/dfi
-    A_wr += d * fi;
-    A_rcol += d * nrm[c] * restc[c] * nc;
-    A_restc[c] += d * rcol * nrm[c] * nc;
-    const R g = bulk ? R(0) : d * rcol * nrm[c] * restc[c];
-    Sg += g * nc;
-    // Eq. (perturb)
-    A_pamp += q * pert;
-    Sn += q * (Ws[c] * nc * nc + Cs[c]);
-    const R p2 = R(2) * pamp * Ws[c] * q * nc;
-    // Eq. (collision): fi = f + itau (feq - f)
-    const R A_feq = q * itau;
-    Af[i] = q * (R(1) - itau);
-    A_itau += q * (feq - f[i]);
-    // Eq. (feq): feq = rwc (cu (9/2 cu + 3) - 3/2 u^2) + restc
-    A_rwc[c] += A_feq * poly;
-    A_restc[c] += A_feq;
-    const R A_cu = A_feq * rwc[c] * (R(9) * cu + R(3));
-    A_uu15 -= A_feq * rwc[c];
-    if (L::ca(i) > 0) { Aua += A_cu; Pa += p2; Ga += g; }
-    if (L::ca(i) < 0) { Aua -= A_cu; Pa -= p2; Ga -= g; }
-    if (L::cb(i) > 0) { Aub += A_cu; Pb += p2; Gb += g; }
-    if (L::cb(i) < 0) { Aub -= A_cu; Pb -= p2; Gb -= g; }
-    if (L::cm(i) > 0) { Aum += A_cu; Pm += p2; Gm += g; }
-    if (L::cm(i) < 0) { Aum -= A_cu; Pm -= p2; Gm -= g; }
-  }
-  // restc_s = rho (A_s + B_s abar), rwc_s = rho W_s
-  R A_rho = R(0), A_abar = R(0);
+      for (int k = 0; k < 3; ++k) {
+        if (!L::D3 && k == 1) continue;
+        uUV = fma(u[k], UV[s][k], uUV);
+        uQV = fma(u[k], QV[s][k], uQV);
+        uDV = fma(u[k], DV[s][k], uDV);
+        eDV = fma(e[k], DV[s][k], eDV);
+        ePV = fma(e[k], PV[s][k], ePV);
+      }
+      // Eq. (feq): sums of q and d times rho W (9/2 (c.u)^2 + 3 c.u - 3/2 u^2)
+      qpoly = fma(R(4.5), uUV, fma(R(3), uQV, qpoly));
+      dpoly = fma(R(4.5), DU[s], fma(R(3), uDV, dpoly));
+      // Eq. (recolor): rcol nrm restc (c.e)
+      A_rcol = fma(nrm * restc, eDV, A_rcol);
+      A_rest = fma(rcol * nrm, eDV, A_rest);
+      const R kg = rdir * nrm * restc;
+      Sg = fma(kg, eDV, Sg);
+      const R rwt = itau * rw;
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    A_rho += A_restc[c] * (As[c] + Bs[c] * abar) + A_rwc[c] * Ws[c];
-    A_abar += A_restc[c] * rho * Bs[c];
+      for (int k = 0; k < 3; ++k) {
+        if (!L::D3 && k == 1) continue;
+        G[k] = fma(kg, DV[s][k], G[k]);
+        P[k] = fma(R(2) * W, PV[s][k], P[k]);
+        Au[k] = fma(rwt, fma(R(9), UV[s][k], R(3) * QV[s][k]), Au[k]);
+      }
+      // Eq. (perturb): |F| (W (c.e)^2 - C)
+      Sn = fma(W, ePV, Sn);
+      Spert_q = fma(W, ePV, Spert_q);
+      Spert_d = fma(W, DN[s], Spert_d);
+    }
+    Sn = fma(C, Q0[s], Sn);
+    Spert_q = fma(-C, Q0[s], Spert_q);
+    Spert_d = fma(-C, D0[s], Spert_d);
+    Sqeq = fma(rw, qpoly, fma(restc, Q0[s], Sqeq));
+    Sdeq = fma(rw, dpoly, fma(restc, D0[s], Sdeq));
+    A_uu15 = fma(-itau * rw, Q0[s], A_uu15);
+    // restc = rho (A + B abar), rw = rho W
+    A_rho = fma(A_rest, rest1, fma(itau * qpoly, W, A_rho));
+    A_abar = fma(A_rest, rho * R(L::B(i)), A_abar);
   }
-  A_itau += A_pamp * amp;  // pamp = amp itau
-  R A_wb = R(0);
-  A_wr += A_rcol * beta * wb + A_itau * ir + A_abar * PHYS(R, ph, alpha_r);  // rcol = beta wr wb
-  A_wb += A_rcol * beta * wr + A_itau * ib + A_abar * PHYS(R, ph, alpha_b);
+  const R A_pamp = Fn * Spert_q;
+  // f_i' = f_i + itau (feq_i - f_i) + pamp pert_i;  f^r_i = wr f_i' + recoloring
+  const R A_itau = fma(amp, A_pamp, Sqeq - Sqf);
+  R A_wr = fma(itau, Sdeq - Sdf, fma(pamp, Fn * Spert_d, Sdf));
+  A_wr = fma(A_rcol, beta * wb, fma(A_itau, ir, fma(A_abar, PHYS(R, ph, alpha_r), A_wr)));
+  const R A_wb = fma(A_rcol, beta * wr, fma(A_itau, ib, A_abar * PHYS(R, ph, alpha_b)));
   // u = j / rho, uu15 = 3/2 |u|^2
-  Aua += R(3) * A_uu15 * ua;
-  Aub += R(3) * A_uu15 * ub;
-  Aum += R(3) * A_uu15 * um;
-  A_rho -= (Aua * ua + Aub * ub + Aum * um) * irho;
-  const R Aja = Aua * irho, Ajb = Aub * irho, Ajm = Aum * irho;
-  // dL/dF = P - pamp Sn e + (G - Sg e) / |F|, e = F / |F| (zero where F = 0, as in the step)
-  const R ea = Fa * iFn, eb = Fb * iFn, em = Fm * iFn;
-  const R se = pamp * Sn + Sg * iFn;
-  lF[0] = Pa + Ga * iFn - se * ea;
-  lF[1] = Pb + Gb * iFn - se * eb;
-  lF[2] = Pm + Gm * iFn - se * em;
-  // wr = rr / rho, wb = rb / rho, rho = rr + rb
-  const R A_rr = A_rho + (A_wr - A_wb) * wb * irho;
-  const R A_rb = A_rho + (A_wb - A_wr) * wr * irho;
+  R Aj[3], Auu = R(0);
 #pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    R a = Af[i];
-    if (L::ca(i) > 0) a += Aja;
-    if (L::ca(i) < 0) a -= Aja;
-    if (L::cb(i) > 0) a += Ajb;
-    if (L::cb(i) < 0) a -= Ajb;
-    if (L::cm(i) > 0) a += Ajm;
-    if (L::cm(i) < 0) a -= Ajm;
-    lg_out(i, V2<R>{a + A_rr, a + A_rb});
+  for (int k = 0; k < 3; ++k) {
+    const R a = fma(R(3) * A_uu15, u[k], Au[k]);
+    Auu = fma(a, u[k], Auu);
+    Aj[k] = a * irho;
   }
+  A_rho = fma(-Auu, irho, A_rho);
+  // dL/dF = 2 pamp sum W q (c.e) c - pamp Sn e + (G - Sg e) / |F| (zero where F = 0)
+  const R se = fma(pamp, Sn, Sg * iFn);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) lF[k] = fma(pamp, P[k], fma(G[k], iFn, -se * e[k]));
+  // wr = rr / rho, wb = rb / rho, rho = rr + rb
+  const R A_rr = fma((A_wr - A_wb) * wb, irho, A_rho);
+  const R A_rb = fma((A_wb - A_wr) * wr, irho, A_rho);
+  const R keep = R(1) - itau;
+  lg_out.each([&](int i) -> V2<R> {
+    R a = keep * q[i];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int c = axis_comp<L>(i, k);
+      if (c) a = c > 0 ? a + Aj[k] : a - Aj[k];
+    }
+    return {a + A_rr, a + A_rb};
+  });
 }
 
-// Kernel A's per-cell tail (replaces StepEpilogue in step_tile).  It reads lambda^{n+1} and
+// lg_i goes where the pull read g_i from: slot i of x - c_i, or slot opp(i) of x for a bounced link
+// (element index in 32 bits: a state holds Q nstore < 2^31 vec2).
+template <int Q, class R, class Vec>
+struct PullPush {
+  Vec* out;
+  int ns, si, lo, hi;
+  int4 to;
+  uint32_t bits;
+  template <class V>
+  __device__ __forceinline__ void each(const V& value) const {
+    using L = Lattice<Q>;
+    if (bits == 0) {
+#pragma unroll
+      for (int i = 0; i < Q; ++i) put(i * ns + pull_source<L>(to, lo, hi, si, i), value(i));
+    } else {
+#pragma unroll
+      for (int i = 0; i < Q; ++i)
+        put((bits >> i) & 1u ? opp(i) * ns + si : i * ns + pull_source<L>(to, lo, hi, si, i), value(i));
+    }
+  }
+  __device__ __forceinline__ void put(int at, V2<R> v2) const {
+    Vec v;
+    v.x = v2.r;
+    v.y = v2.b;
+    out[at] = v;
+  }
+};
+
+// Kernel A's per-cell tail (in the place of PairStep in pair_tile).  It reads lambda^{n+1} and
 // writes the transpose of the pull of step n directly:
 //   lambda^n_j(y) = lg_j(y + c_j) + ab(y + c_j), or lg_{opp j}(y) + ab(y) where y + c_j is solid
 // or beyond a wall, with ab = mu d rho^N / d(rho_r, rho_b) from kernel B1 of the same step.  Its
@@ -254,6 +330,8 @@ struct AdjointEpilogue {
     const int bx = (int)threadIdx.x % TX + 1;
     const int by = L::D3 ? (int)threadIdx.x / TX + 1 : 0;
     const Vec* box = reinterpret_cast<const Vec*>(abox);
+    const Vec* const here[3] = {box + ((m - 1) & 3) * NB + by * BX + bx, box + (m & 3) * NB + by * BX + bx,
+                                box + ((m + 1) & 3) * NB + by * BX + bx};
     async_wait_all();  // this thread's copies of plane m (only it reads its column)
     const Vec* col = reinterpret_cast<const Vec*>(lam);
     auto lam_at = [&](int i) -> V2<R> {
@@ -261,19 +339,10 @@ struct AdjointEpilogue {
       // ab of the slot's writer: x = y + c_i, or y itself where y + c_i is solid (the source of
       // this cell's direction opp(i))
       const bool self = i == 0 || ((sbits >> opp(i)) & 1u);
-      const Vec w = self ? box[(m & 3) * NB + by * BX + bx]
-                         : box[((m + L::cm(i)) & 3) * NB + (by + L::cb(i)) * BX + bx + L::ca(i)];
+      const Vec w = *(self ? here[1] : here[1 + L::cm(i)] + L::cb(i) * BX + L::ca(i));
       return {v.x + w.x, v.y + w.y};
     };
-    auto lg_out = [&](int i, V2<R> v2) {
-      Vec v;
-      v.x = v2.r;
-      v.y = v2.b;
-      // element index in 32 bits (a state holds Q nstore < 2^31 vec2)
-      const bool bounce = (sbits >> i) & 1u;
-      const int idx = bounce ? opp(i) * ns + si : i * ns + pull_source<L>(to, pm.lo, pm.hi, si, i);
-      lout[idx] = v;
-    };
+    const PullPush<Q, R, Vec> lg_out{lout, ns, si, pm.lo, pm.hi, to, sbits};
     R lF[3];
     R Fa, Fb, Fm;
     colour_gradient<Q, R>(rnb, Fa, Fb, Fm);
@@ -288,7 +357,7 @@ struct AdjointEpilogue {
 };
 
 template <int Q, int S, int TX, int TY>
-__global__ void __launch_bounds__(TX* TY, (S == ST_F64 ? 256 : 384) / (TX * TY))
+__global__ void __launch_bounds__(TX* TY, (S == ST_F64 ? 256 : ADJ_T) / (TX * TY))
     cg_adjoint_local_kernel(const __grid_constant__ StepArgs A,
                             const __grid_constant__ AdjointOut O) {
   extern __shared__ __align__(16) unsigned char dyn_smem[];
@@ -301,7 +370,71 @@ __global__ void __launch_bounds__(TX* TY, (S == ST_F64 ? 256 : 384) / (TX * TY))
   constexpr int lam_bytes = Q * TX * TY * (int)sizeof(Vec);
   unsigned char* const lam0 = dyn_smem + PairSmem<Q, S, TX, TY>::BYTES;
   const Epi E{O, lam0 + threadIdx.x * sizeof(Vec), lam0 + lam_bytes};
-  pair_tile<Q, S, TX, TY, true, true>(A, blockIdx.x, blockIdx.y, dyn_smem, n, d, threadIdx.x, E, CtaSync());
+  pair_tile<Q, S, TX, TY, ADJ_PF, true>(A, blockIdx.x, blockIdx.y, dyn_smem, n, d, threadIdx.x, E, CtaSync());
+}
+
+// (2) one thread per cell.  dLdV: pointer to dL/dV(n+1) (nullptr: 0).  The kernel was bound by its
+// integer instructions (47 % of them; two divisions a cell for the coordinates), so the coordinates
+// come from the launch: blocks of kStencilX x 256 / kStencilX cells of a plane (a row in 2D), planes
+// along grid z, both strided where the grid is smaller than the lattice.
+template <int Q>
+__host__ __device__ constexpr int stencil_x() { return Q == 19 ? 64 : 256; }
+
+template <int Q, class R>
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 8 : 5)  // FP32: 32 registers, all warps resident
+    cg_adjoint_stencil_kernel(Geom G, const R* __restrict__ aux, const void* __restrict__ lam_g,
+                              void* __restrict__ ab, const uint8_t* __restrict__ mask,
+                              double* __restrict__ dphi, double inv_sbar,
+                              const double* __restrict__ dLdV) {
+  using L = Lattice<Q>;
+  using Vec = typename std::conditional<sizeof(R) == 8, double2, float2>::type;
+  constexpr int BX = stencil_x<Q>(), BY = 256 / BX;
+  const int a = blockIdx.x * BX + threadIdx.x % BX;
+  if (a >= G.na) return;
+  const R w0 = dLdV ? R(0.5 * __ldg(dLdV)) : R(0);
+  for (int m = blockIdx.z; m < G.nm; m += gridDim.z)
+    for (int b = blockIdx.y * BY + threadIdx.x / BX; b < G.nb; b += gridDim.y * BY) {
+      const int cell = (m * G.nb + b) * G.na + a;
+      const Slot sl = make_slot<L>(G, a, b);
+      const Plane p = make_plane(G, m);
+      uint32_t bits = 0;
+      if (!solid_bits<L>(G, sl, p, cell, bits)) continue;
+      const PlaneOffsets po = plane_offsets(G, m);
+      const int4 to = make_int4(sl.dxm, sl.dxp, sl.dym, sl.dyp);
+      const int si = sidx(G, a, b, m);
+      const int ns = G.nstore;  // 5 ns < Q nstore < 2^31
+      const R oa = aux[si], ob = aux[ns + si], om = aux[2 * ns + si];
+      R mu = w0;
+      auto from = [&](int i) {  // F of x = y - c_i used rho^N(y) with weight 3 W_i c_i
+        const int src = pull_source<L>(to, po.dm_lo, po.dm_hi, si, i);
+        R t = R(0);
+        if (L::ca(i)) t += R(L::ca(i)) * __ldg(aux + src);
+        if (L::cb(i)) t += R(L::cb(i)) * __ldg(aux + (ns + src));
+        if (L::cm(i)) t += R(L::cm(i)) * __ldg(aux + (2 * ns + src));
+        return t;
+      };
+      if (bits == 0) {
+#pragma unroll
+        for (int i = 1; i < Q; ++i) mu += R(3.0 * L::W(i)) * from(i);
+      } else {
+#pragma unroll
+        for (int i = 1; i < Q; ++i) {
+          R t = R(0);
+          if (!((bits >> i) & 1u)) t = from(i);  // x = y - c_i is fluid
+          if ((bits >> opp(i)) & 1u)  // y + c_i is solid: y's own F used rho^N(y) in its place
+            t += R(L::ca(i)) * oa + R(L::cb(i)) * ob + R(L::cm(i)) * om;
+          mu += R(3.0 * L::W(i)) * t;
+        }
+      }
+      Vec v;
+      v.x = mu * aux[3 * ns + si];
+      v.y = mu * aux[4 * ns + si];
+      reinterpret_cast<Vec*>(ab)[si] = v;
+      if (mask[cell] & 1u) {  // Eq. (exchange): d g_0^r / d phi = -1/S-bar, d g_0^b / d phi = +1/S-bar
+        const Vec l0 = reinterpret_cast<const Vec*>(lam_g)[si];
+        dphi[cell] += ((double)(l0.y + v.y) - (double)(l0.x + v.x)) * inv_sbar;
+      }
+    }
 }
 
 __device__ __forceinline__ void cell_coords(const Geom& g, int cell, int& a, int& b, int& m) {
@@ -309,52 +442,6 @@ __device__ __forceinline__ void cell_coords(const Geom& g, int cell, int& a, int
   const int t = cell / g.na;
   b = t % g.nb;
   m = t / g.nb;
-}
-
-// (2) one thread per cell.  dLdV: pointer to dL/dV(n+1) (nullptr: 0).
-template <int Q, class R>
-__global__ void __launch_bounds__(256)
-    cg_adjoint_stencil_kernel(Geom G, const R* __restrict__ aux, const void* __restrict__ lam_g,
-                              void* __restrict__ ab, const uint8_t* __restrict__ mask,
-                              double* __restrict__ dphi, double inv_sbar,
-                              const double* __restrict__ dLdV) {
-  using L = Lattice<Q>;
-  using Vec = typename std::conditional<sizeof(R) == 8, double2, float2>::type;
-  const int cell = blockIdx.x * blockDim.x + threadIdx.x;
-  if (cell >= G.ncell) return;
-  int a, b, m;
-  cell_coords(G, cell, a, b, m);
-  const Slot sl = make_slot<L>(G, a, b);
-  const Plane p = make_plane(G, m);
-  uint32_t bits = 0;
-  if (!solid_bits<L>(G, sl, p, cell, bits)) return;
-  const PlaneOffsets po = plane_offsets(G, m);
-  const int4 to = make_int4(sl.dxm, sl.dxp, sl.dym, sl.dyp);
-  const int si = sidx(G, a, b, m);
-  const size_t ns = G.nstore;
-  const R oa = aux[si], ob = aux[ns + si], om = aux[2 * ns + si];
-  R mu = dLdV ? R(0.5 * __ldg(dLdV)) : R(0);
-#pragma unroll
-  for (int i = 1; i < Q; ++i) {
-    R t = R(0);
-    if (!((bits >> i) & 1u)) {  // x = y - c_i is fluid: its F used rho^N(y) with weight 3 W_i c_i
-      const int src = pull_source<L>(to, po.dm_lo, po.dm_hi, si, i);
-      if (L::ca(i)) t += R(L::ca(i)) * __ldg(aux + src);
-      if (L::cb(i)) t += R(L::cb(i)) * __ldg(aux + ns + src);
-      if (L::cm(i)) t += R(L::cm(i)) * __ldg(aux + 2 * ns + src);
-    }
-    if ((bits >> opp(i)) & 1u)  // y + c_i is solid: y's own F used rho^N(y) in its place
-      t += R(L::ca(i)) * oa + R(L::cb(i)) * ob + R(L::cm(i)) * om;
-    mu += R(3.0 * L::W(i)) * t;
-  }
-  Vec v;
-  v.x = mu * aux[3 * ns + si];
-  v.y = mu * aux[4 * ns + si];
-  reinterpret_cast<Vec*>(ab)[si] = v;
-  if (mask[cell] & 1u) {  // Eq. (exchange): d g_0^r / d phi = -1/S-bar, d g_0^b / d phi = +1/S-bar
-    const Vec l0 = reinterpret_cast<const Vec*>(lam_g)[si];
-    dphi[cell] += ((double)(l0.y + v.y) - (double)(l0.x + v.x)) * inv_sbar;
-  }
 }
 
 // V = sum over fluid cells of (1 + rho^N)/2 of a stored state, FP64, deterministic: fixed grid,

@@ -1,5 +1,7 @@
 // adjoint_kernels.cu -- instantiations and launchers of the adjoint sweep and of the volume
 // observable (adjoint.cuh).
+#include <algorithm>
+
 #include "adjoint.cuh"
 #include "launch.h"
 
@@ -46,7 +48,9 @@ cudaError_t launch_adjoint_stencil(const AuxArgs& a, const void* aux, const void
                                    const uint8_t* mask, double* dphi, double inv_sbar,
                                    const double* dLdV, cudaStream_t s) {
   if (a.g.ncell <= 0) return cudaSuccess;
-  const unsigned nb = blocks_for(a.g.ncell);
+  const int bx = a.q == 19 ? stencil_x<19>() : stencil_x<9>(), by = 256 / bx;
+  const dim3 nb((unsigned)((a.g.na + bx - 1) / bx), (unsigned)std::min((a.g.nb + by - 1) / by, 65535),
+                (unsigned)std::min(a.g.nm, 65535));
   if (a.q == 19 && a.storage == ST_F64)
     cg_adjoint_stencil_kernel<19, double><<<nb, kThreads, 0, s>>>(
         a.g, (const double*)aux, lam_g, ab, mask, dphi, inv_sbar, dLdV);

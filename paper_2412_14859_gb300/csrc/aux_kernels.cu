@@ -87,21 +87,24 @@ __global__ void k_init_eq(Geom g, Physics ph, double rri, double rbi, const doub
     double fr[Q], fb[Q];
     const bool solid = cell_solid(g, cell);
     const double rn = rhoN0[cell];
-    const double rr = rri * (1.0 + rn) / 2.0, rb = rbi * (1.0 - rn) / 2.0;
+    const double rr = solid ? 0.0 : rri * (1.0 + rn) / 2.0, rb = solid ? 0.0 : rbi * (1.0 - rn) / 2.0;
+    // a speed class's directions start alike: without noise one product and one conversion to the
+    // storage's type per class, where one per direction held the kernel to the FP64 rate
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-      if (solid) {
-        fr[i] = fb[i] = 0.0;
-        continue;
-      }
       fr[i] = rr * (L::A(i) + L::B(i) * ph.alpha_r);
       fb[i] = rb * (L::A(i) + L::B(i) * ph.alpha_b);
-      if (noise) {
+    }
+    if (noise && !solid) {
+#pragma unroll
+      for (int i = 0; i < Q; ++i) {
         fr[i] += read_any(noise, ndt, (size_t)i * g.ncell + cell);
         fb[i] += read_any(noise, ndt, (size_t)(Q + i) * g.ncell + cell);
       }
+      store_cell<Q, S>(state, g, cell, fr, fb, ph);
+    } else {
+      store_cell<Q, S>(state, g, cell, fr, fb, ph);
     }
-    store_cell<Q, S>(state, g, cell, fr, fb, ph);
   }
 }
 
@@ -140,26 +143,31 @@ __global__ void k_macros(Geom g, Physics ph, const void* state, double* rr_out, 
   for (int cell = blockIdx.x * blockDim.x + threadIdx.x; cell < g.ncell; cell += gridDim.x * blockDim.x) {
     double fr[Q], fb[Q];
     load_cell<Q, S>(state, g, cell, fr, fb, ph);
-    double rr = 0, rb = 0, ja = 0, jb = 0, jm = 0;
+    // bound by the FP64 rate: momenta from the differences of opposite directions, no products with
+    // c, one division a cell
+    double rr = fr[0], rb = fb[0], ja = 0, jb = 0, jm = 0;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      rr += fr[i];
-      rb += fb[i];
-      const double f = fr[i] + fb[i];
-      ja += L::ca(i) * f;
-      jb += L::cb(i) * f;
-      jm += L::cm(i) * f;
+    for (int i = 1; i < Q; i += 2) {
+      rr += fr[i] + fr[i + 1];
+      rb += fb[i] + fb[i + 1];
+      if (u_out) {
+        const double d = (fr[i] - fr[i + 1]) + (fb[i] - fb[i + 1]);
+        if (L::ca(i)) ja += L::ca(i) > 0 ? d : -d;
+        if (L::cb(i)) jb += L::cb(i) > 0 ? d : -d;
+        if (L::cm(i)) jm += L::cm(i) > 0 ? d : -d;
+      }
     }
     const double rho = rr + rb;
+    const double irho = 1.0 / rho;
     const bool solid = cell_solid(g, cell) || !(rho > 0.0);
     if (rr_out) rr_out[cell] = solid ? 0.0 : rr;
     if (rb_out) rb_out[cell] = solid ? 0.0 : rb;
-    if (rn_out) rn_out[cell] = solid ? 0.0 : (rr - rb) / rho;
+    if (rn_out) rn_out[cell] = solid ? 0.0 : (rr - rb) * irho;
     if (u_out) {
       // (a, b, m) -> (x, y, z): 3D (x, y, z); 2D (x, -, y)
-      const double ux = solid ? 0.0 : ja / rho;
-      const double uy = solid ? 0.0 : (L::D3 ? jb : jm) / rho;
-      const double uz = solid ? 0.0 : (L::D3 ? jm : 0.0) / rho;
+      const double ux = solid ? 0.0 : ja * irho;
+      const double uy = solid ? 0.0 : (L::D3 ? jb : jm) * irho;
+      const double uz = solid ? 0.0 : (L::D3 ? jm : 0.0) * irho;
       u_out[cell] = ux;
       u_out[(size_t)g.ncell + cell] = uy;
       u_out[2 * (size_t)g.ncell + cell] = uz;
