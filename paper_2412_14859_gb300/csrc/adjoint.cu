@@ -68,8 +68,7 @@ int launch_step_on(cgevap_sim* s, const void* pin, void* pout, const uint8_t* ma
   a.mask_out = mask_out;
   a.red.ledger = ledger;
   void* args[] = {&a};
-  CG_CUDA(s, cudaLaunchKernel(step_fn(s->kernel, a), dim3(s->ntx * s->nty, s->nchunk),
-                              dim3(s->kernel.threads), args, s->kernel.smem, s->stream));
+  CG_CUDA(s, launch_step(s->kernel, a, dim3(s->ntx * s->nty, s->nchunk), args, s->stream));
   return CGEVAP_OK;
 }
 

@@ -26,12 +26,6 @@
 #include "launch.h"
 #include "pair_tile.cuh"
 
-#ifndef ADJ_T
-#define ADJ_T 384
-#endif
-#ifndef ADJ_PF
-#define ADJ_PF true
-#endif
 namespace cgevap {
 
 // Minority fraction product w_r w_b below which the adjoint holds the recoloring direction fixed.
@@ -357,7 +351,7 @@ struct AdjointEpilogue {
 };
 
 template <int Q, int S, int TX, int TY>
-__global__ void __launch_bounds__(TX* TY, (S == ST_F64 ? 256 : ADJ_T) / (TX * TY))
+__global__ void __launch_bounds__(TX* TY, (S == ST_F64 ? 256 : 384) / (TX * TY))
     cg_adjoint_local_kernel(const __grid_constant__ StepArgs A,
                             const __grid_constant__ AdjointOut O) {
   extern __shared__ __align__(16) unsigned char dyn_smem[];
@@ -370,7 +364,7 @@ __global__ void __launch_bounds__(TX* TY, (S == ST_F64 ? 256 : ADJ_T) / (TX * TY
   constexpr int lam_bytes = Q * TX * TY * (int)sizeof(Vec);
   unsigned char* const lam0 = dyn_smem + PairSmem<Q, S, TX, TY>::BYTES;
   const Epi E{O, lam0 + threadIdx.x * sizeof(Vec), lam0 + lam_bytes};
-  pair_tile<Q, S, TX, TY, ADJ_PF, true>(A, blockIdx.x, blockIdx.y, dyn_smem, n, d, threadIdx.x, E, CtaSync());
+  pair_tile<Q, S, TX, TY, true, true>(A, blockIdx.x, blockIdx.y, dyn_smem, n, d, threadIdx.x, E, CtaSync());
 }
 
 // (2) one thread per cell.  dLdV: pointer to dL/dV(n+1) (nullptr: 0).  The kernel was bound by its

@@ -170,6 +170,17 @@ int plan_launch(cgevap_sim* s, int family, int variant, int pc_force = 0) {
   KernelRef k = family == 1 ? step_tma_f32(s->p.q, variant)
                             : kernel_for(s->p.q, s->p.storage, variant);
   if (!k.fn) return fail(s, CGEVAP_ERR_UNSUPPORTED, "no step kernel for this configuration");
+  // the default D2Q9 step of the pair storages does not march (cgevap_tune with planes_per_chunk or
+  // another variant does)
+  bool patch = false;
+  if (family == 0 && variant == 0 && pc_force == 0 && s->p.q == 9) {
+    KernelRef flat{nullptr, 0};
+    if (s->p.storage == CGEVAP_F64) flat = patch_kernel_f64(s->N);
+    if (s->p.storage == CGEVAP_F32 || s->p.storage == CGEVAP_F32X)
+      flat = patch_kernel_f32(internal_storage(s->p.storage), s->N);
+    patch = flat.fn && (s->geom.nm + flat.ty - 1) / flat.ty <= 65535;
+    if (patch) k = flat;
+  }
   KernelRef k_in{nullptr, 0};
   if (is_recolour_on_pull(s->p.storage)) {  // same tiles, FP32 pairs in
     k_in = kernel_for(s->p.q, s->p.storage, variant, true);
@@ -183,7 +194,7 @@ int plan_launch(cgevap_sim* s, int family, int variant, int pc_force = 0) {
   if (occ < 1) occ = 1;
   const int na = s->geom.na, nb = s->geom.nb, nm = s->geom.nm;
   const int ntx = (na + t.tx - 1) / t.tx;
-  const int nty = (nb + t.ty - 1) / t.ty;
+  const int nty = patch ? 1 : (nb + t.ty - 1) / t.ty;
   const long long tiles = (long long)ntx * nty;
   const long long slots = (long long)occ * sms;
   int best_pc = nm;
@@ -200,6 +211,7 @@ int plan_launch(cgevap_sim* s, int family, int variant, int pc_force = 0) {
     }
   }
   if (pc_force > 0) best_pc = pc_force < nm ? pc_force : nm;
+  if (patch) best_pc = t.ty;  // rows of a patch
   if (k.needs_map) {
     const int bh = s->p.q == 19 ? t.ty + 2 : 1;
     for (int h = 0; h < 2; ++h) {
@@ -251,6 +263,7 @@ StepArgs cgevap::step_args(cgevap_sim* s) {
   a.red.done = s->done;
   a.red.ledger = s->ledger;
   a.red.status = s->status;
+  a.red.tally = s->tally;
   a.ntx = s->ntx;
   a.nty = s->nty;
   a.pc = s->pc;
@@ -283,8 +296,7 @@ int launch_one_step(cgevap_sim* s) {
   StepArgs a = step_args(s);
   void* args[] = {&a, s->tmap[s->cur]};
   const KernelRef& k = s->rc_pairs && s->kernel_in.fn ? s->kernel_in : s->kernel;
-  CG_CUDA(s, cudaLaunchKernel(step_fn(k, a), dim3(s->ntx * s->nty, s->nchunk), dim3(k.threads), args, k.smem,
-                              s->stream));
+  CG_CUDA(s, launch_step(k, a, dim3(s->ntx * s->nty, s->nchunk), args, s->stream));
   s->cur ^= 1;
   s->rc_pairs = 0;
   return CGEVAP_OK;
@@ -311,7 +323,7 @@ void release(cgevap_sim* s) {
   adjoint_release(s);
   void* ptrs[] = {s->state[0], s->state[1], s->mask[0],  s->mask[1],  s->links,
                   s->solid,    s->phi_field, s->ledger, s->part_removed, s->part_sites,
-                  s->done,     s->tmp_rn,   s->flag,    s->staging, s->status,
+                  s->done,     s->tmp_rn,   s->flag,    s->staging, s->status, s->tally,
                   s->vol_part, s->vol_done, s->heat.part};
   for (void* q : ptrs)
     if (q) cudaFree(q);
@@ -394,7 +406,8 @@ int cgevap_create(const cgevap_params* p, cgevap_sim** out) {
   ok = ok && cudaMalloc(&s->ledger, sizeof(DevLedger)) == cudaSuccess &&
        cudaMalloc(&s->done, sizeof(unsigned int)) == cudaSuccess &&
        cudaMalloc(&s->flag, sizeof(int)) == cudaSuccess &&
-       cudaMalloc(&s->status, sizeof(int)) == cudaSuccess;
+       cudaMalloc(&s->status, sizeof(int)) == cudaSuccess &&
+       cudaMalloc(&s->tally, sizeof(unsigned long long)) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
     release(s);
@@ -406,7 +419,8 @@ int cgevap_create(const cgevap_params* p, cgevap_sim** out) {
            cudaMemset(s->mask[1], 0, s->N) == cudaSuccess &&
            cudaMemset(s->ledger, 0, sizeof(DevLedger)) == cudaSuccess &&
            cudaMemset(s->done, 0, sizeof(unsigned int)) == cudaSuccess &&
-           cudaMemset(s->status, 0, sizeof(int)) == cudaSuccess;
+           cudaMemset(s->status, 0, sizeof(int)) == cudaSuccess &&
+           cudaMemset(s->tally, 0, sizeof(unsigned long long)) == cudaSuccess;
   if (!z) {
     release(s);
     return fail(nullptr, CGEVAP_ERR_CUDA, "initial memset failed");

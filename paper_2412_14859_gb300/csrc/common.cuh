@@ -113,6 +113,8 @@ struct Reduce {
   unsigned int* done;            // arrival counter, returned to 0 by the last block
   DevLedger* ledger;
   int* status;                   // set to 1 by a bounded wait that gave up (may be nullptr)
+  unsigned long long* tally;     // arrivals and sites of a step in one word, 0 between steps
+                                 // (cg_patch_kernel; nullptr for callers that do not run it)
 };
 
 struct StepArgs {

@@ -29,15 +29,33 @@ struct KernelRef {
   int smem = 0;       // dynamic shared memory bytes
   int tx = 0, ty = 0; // tile shape (0: take it from tile_cfg)
   int needs_map = 0;  // 1: second kernel argument is the TMA tensor map of the input state
+  int pdl = 0;                  // 1: may be launched ahead of its predecessor's end (it waits itself)
   const void* plain = nullptr;  // the same step without links, site bytes read or a flux field
 };
 // The instantiation that runs step arguments a.
 inline const void* step_fn(const KernelRef& k, const StepArgs& a) {
   return k.plain && !a.g.links && a.ph.rule == 1 && !a.ph.phi_field ? k.plain : k.fn;
 }
+// Launches a step kernel; a kernel that waits for its predecessor itself is launched ahead of it.
+inline cudaError_t launch_step(const KernelRef& k, const StepArgs& a, dim3 grid, void** args, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)k.threads);
+  cfg.dynamicSmemBytes = (size_t)k.smem;
+  cfg.stream = s;
+  cudaLaunchAttribute ahead;
+  ahead.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  ahead.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &ahead;
+  cfg.numAttrs = k.pdl ? 1u : 0u;
+  return cudaLaunchKernelExC(&cfg, step_fn(k, a), args);
+}
 KernelRef step_kernel_f64(int q, int variant);
 KernelRef step_kernel_f32(int q, int variant);
 KernelRef step_kernel_f32x(int q, int variant);  // FP32 pairs, exact colour masses (step_f32.cu)
+// D2Q9 step of the pair storages without a march (pair_tile.cuh), for a lattice of that many cells.
+KernelRef patch_kernel_f64(long long cells);
+KernelRef patch_kernel_f32(int storage, long long cells);  // ST_F32 or ST_F32X
 KernelRef step_kernel_dev(int q, int storage, int variant);
 // Recolour-on-pull layout (step_rc.cu); pairs_in: the input state holds FP32 pairs (import).
 KernelRef step_kernel_rc(int q, int variant, bool pairs_in);

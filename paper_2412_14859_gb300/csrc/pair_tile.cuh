@@ -123,7 +123,10 @@ __device__ __forceinline__ double recip_density(double x) {
 // y (1 + e/2 + 3 e^2/8) with e = 1 - F2 y^2; outside the range the approximation holds for, the
 // square root and the division (GB300 issues an FP64 instruction every 16 cycles a warp: 7 of
 // them here against about 25).
-__device__ __forceinline__ void norm_of(float F2, float& Fn, float& iFn) { norm_pair<float>(F2, Fn, iFn); }
+__device__ __forceinline__ void norm_of(float F2, float& Fn, float& iFn) {
+  iFn = rsqrtf(F2);
+  Fn = mul_rn(F2, iFn);
+}
 __device__ __forceinline__ void norm_of(double F2, double& Fn, double& iFn) {
   if (F2 > 1e-280 && F2 < 1e280) {
     double y;
@@ -191,6 +194,21 @@ __device__ __forceinline__ typename Storage<S>::real exchange_sums(
   rb = sb + e;
   flags = (site ? 1u : 0u) | (near ? 4u : 0u);
   return ALT ? fma(sr - sb, irho, -mul_rn(R(2) * e, irho)) : fma(R(-2) * e, irho, rn_pre);
+}
+
+// ST_F32X: the rounding errors (lr, lb) of a cell's post-exchange totals rr, rb: what the colour
+// totals summed without rounding error (from B) exceed the plain sums sr, sb by, and the exchange's
+// own rounding (TwoSum).
+template <int Q>
+__device__ __forceinline__ void exact_errors(const Physics& ph, const V2<float> (&g)[Q], float sr, float sb,
+                                             float rr, float rb, float e, float& lr, float& lb) {
+  float2 acc = sum_start(ph), lo = make_float2(0.0f, 0.0f);
+#pragma unroll
+  for (int i = 0; i < Q; ++i) fast_two_sum_acc(acc, lo, make_float2(g[i].r, g[i].b));
+  // (acc - B) and the plain sums are both within a few ulps of B of the total: exact difference
+  lo = __fadd2_rn(sub2(sub2(acc, sum_start(ph)), make_float2(sr, sb)), lo);
+  lr = __fadd_rn(lo.x, two_sum_err(sr, -e, rr));
+  lb = __fadd_rn(lo.y, two_sum_err(sb, e, rb));
 }
 
 // Sum of s_p v_p over the pairs p of opposite directions (i, i + 1) with c_i = s along an axis
@@ -309,8 +327,9 @@ __device__ __forceinline__ float collide_pairs(const Physics& ph, const CellMome
     kr[c] = rcol * iFn * R(inv_norm<L>(i)) * restc[c];
   }
   const R f0eq = fma(rwc[0], -uu15, restc[0]);
-  const R fi0 = fma(itau, f0eq - f[0], f[0]) - kc[0];
-  out(0, wr * fi0, fi0 - wr * fi0);
+  const R fi0 = fma(-mul_rn(pamp, R(L::C(0))), Fn, fma(itau, f0eq - f[0], f[0]));
+  const R r0 = mul_rn(wr, fi0);
+  out(0, r0, fi0 - r0);
 #pragma unroll
   for (int i = 1; i < Q; i += 2) {
     const int j = i + 1;
@@ -401,6 +420,15 @@ __device__ __forceinline__ double collide_pairs(const Physics& ph, const CellMom
   }
   return Fn;
 }
+
+// Programmatic dependent launch: a step's launch is prepared while its predecessor runs, and its CTAs
+// wait for the predecessor's end and its writes before they read anything.  dependents_may_start()
+// lets them take their places as soon as every CTA of this step has started: worth it for the short
+// patch kernel (64^2 FP32 with the tally below 7.2 -> 3.3 us a step), not for the march, whose
+// free slots they would fill (192^3 362 us without, 388 with it).  Without the launch attribute both
+// are no-ops.
+__device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // The barrier of a tile's threads, between the writes and the reads of a plane's rho^N.
 struct CtaSync {  // a whole CTA
@@ -575,7 +603,7 @@ __device__ __forceinline__ void pair_tile(const StepArgs& A, int tile, int chunk
   nxt.flags = 0u;
   nxt.bits = kNoCell;
   int nloc = 0;
-  R rem = R(0);
+  double rem = 0.0;
   // Fill plane um: rho^N of the tile and its ring into slot (um - m0 + 1) & 3, the own cell's
   // sums into park plane (um - m0) & 1.  count: the plane is the chunk's own (its sites count).
   auto fill = [&](int um, bool count, bool more, auto march) {
@@ -613,15 +641,7 @@ __device__ __forceinline__ void pair_tile(const StepArgs& A, int tile, int chunk
       colour_sums<Q, R>(g, sr, sb);
       rn = exchange_sums<S, GEN, decltype(march)::value>(A.ph, mb, phi, sr, sb, nxt.rr, nxt.rb, e, nxt.flags, nxt.irho);
       if constexpr (ExactPairs<S>::value) {
-        // the colour totals without rounding error (from B); what they exceed the plain sums by,
-        // and the exchange's own rounding (TwoSum), go to (lr, lb)
-        float2 acc = sum_start(A.ph), lo = make_float2(0.0f, 0.0f);
-#pragma unroll
-        for (int i = 0; i < Q; ++i) fast_two_sum_acc(acc, lo, make_float2(g[i].r, g[i].b));
-        // (acc - B) and the plain sums are both within a few ulps of B of the total: exact difference
-        lo = __fadd2_rn(sub2(sub2(acc, sum_start(A.ph)), make_float2(sr, sb)), lo);
-        nxt.lr = __fadd_rn(lo.x, two_sum_err(sr, -e, nxt.rr));
-        nxt.lb = __fadd_rn(lo.y, two_sum_err(sb, e, nxt.rb));
+        exact_errors<Q>(A.ph, g, sr, sb, nxt.rr, nxt.rb, e, nxt.lr, nxt.lb);
       }
 #pragma unroll
       for (int i = 0; i < Q; ++i) pk[i * NT] = i == 0 ? (g[0].r - e) + (g[0].b + e) : g[i].r + g[i].b;
@@ -629,7 +649,7 @@ __device__ __forceinline__ void pair_tile(const StepArgs& A, int tile, int chunk
         epi.filled(A, um * pcell + me.cell, nxt.flags);
         if (nxt.flags & 1u) {
           ++nloc;
-          rem += e;
+          rem += (double)e;
         }
       }
     }
@@ -678,7 +698,7 @@ __device__ __forceinline__ void pair_tile(const StepArgs& A, int tile, int chunk
   }
   n_sites = nloc;
   // a scalar flux moves varphi at every site: n varphi in FP64, exact to one rounding
-  removed = A.ph.phi_field ? (double)rem : (double)nloc * A.ph.varphi;
+  removed = A.ph.phi_field ? rem : (double)nloc * A.ph.varphi;
 }
 
 template <int Q, int S, int TX, int TY, int MINB, bool PF, bool GEN>
@@ -686,9 +706,148 @@ __global__ void __launch_bounds__(TX* TY, MINB) cg_pair_kernel(const __grid_cons
   extern __shared__ __align__(16) unsigned char dyn_smem[];
   long long n = 0;
   double d = 0.0;
+  wait_for_previous();
   pair_tile<Q, S, TX, TY, PF, GEN>(A, blockIdx.x, blockIdx.y, dyn_smem, n, d, threadIdx.x, PairStep<GEN>(), CtaSync());
   block_sum<TX * TY>(n, d);
   ledger_fold(A.red, n, d);
+}
+
+// ---- D2Q9 without a march ------------------------------------------------------------------------
+// A plane lattice is small: marched in rows, 64^2 ran three serial fills a step on 64 CTAs (one row
+// each) and 256^2 pulled three rows for each row written.  Here a CTA takes a TX x TY patch and
+// every cell of the patch and of the ring around it has a thread of its own: one round of pulls,
+// one barrier, the collision.  The inner cells come first, so that the warps which collide are full.
+template <int TX, int TY>
+struct PatchShape {
+  static constexpr int NI = TX * TY, HX = TX + 2, HY = TY + 2, NR = HX * HY - NI;
+  static constexpr int THREADS = NI + ((NR + 31) & ~31);
+  static_assert(NI % 32 == 0, "whole warps of inner cells");
+};
+
+template <int S, int TX, int TY, bool GEN>
+__global__ void __launch_bounds__(PatchShape<TX, TY>::THREADS) cg_patch_kernel(const __grid_constant__ StepArgs A) {
+  constexpr int Q = 9;
+  using L = Lattice<Q>;
+  using R = typename Storage<S>::real;
+  using P = PatchShape<TX, TY>;
+  __shared__ R ring[P::HY][P::HX];
+  const Geom& G = A.g;
+  const int tid = threadIdx.x;
+  const bool inner = tid < P::NI;
+  int hx, hy;  // place in the patch with its ring
+  if (inner) {
+    hx = tid % TX + 1;
+    hy = tid / TX + 1;
+  } else {
+    const int k = tid - P::NI;
+    if (k < 2 * P::HX) {
+      hx = k < P::HX ? k : k - P::HX;
+      hy = k < P::HX ? 0 : P::HY - 1;
+    } else {
+      hx = (k & 1) ? P::HX - 1 : 0;
+      hy = 1 + ((k - 2 * P::HX) >> 1);
+    }
+  }
+  const int ua = blockIdx.x * TX + hx - 1, um = blockIdx.y * TY + hy - 1;
+  const bool mine = inner && ua < G.na && um < G.nm;
+  dependents_may_start();
+  R e = R(0);
+  R rr = R(0), rb = R(0), irho = R(0), lr = R(0), lb = R(0), rn = R(0);
+  R f[Q];
+  uint32_t flags = 0u, bits = kNoCell;
+  int si = 0, cell = 0;
+  PairStep<GEN> epi;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) f[i] = R(0);
+  int4 to;
+  March p;
+  wait_for_previous();
+  // ring threads past the ring, and cells beyond the first over a ragged edge, have nothing to do
+  if (tid < P::NI + P::NR && um <= G.nm) {
+    const Column c = make_column<L>(G, ua, 0, to);
+    p = make_march<L>(G, um);
+    if (p.ok && !(c.wall & kNoCell)) {
+      cell = p.m * G.na + c.cell;
+      bits = c.wall | p.wall;
+      if (GEN && G.links) {
+        const uint32_t link = __ldg(G.links + cell);
+        bits = link & kNoCell ? kNoCell : bits | link;
+      }
+    }
+    if (bits != kNoCell) {
+      uint32_t mb = 0u;
+      R phi = R(0);
+      if (GEN && A.ph.rule != 1) mb = A.mask_in[cell];
+      if (GEN && A.ph.phi_field) phi = __ldg(reinterpret_cast<const R*>(A.ph.phi_field) + cell);
+      si = p.m * G.rows * G.pitch + c.col;
+      V2<R> g[Q];
+      pull_pairs<Q, S>(A.pin, G.nstore, to, si, p.lo, p.hi, bits, g);
+      R sr, sb;
+      colour_sums<Q, R>(g, sr, sb);
+      rn = exchange_sums<S, GEN, false>(A.ph, mb, phi, sr, sb, rr, rb, e, flags, irho);
+      if (mine) {
+        if constexpr (ExactPairs<S>::value) exact_errors<Q>(A.ph, g, sr, sb, rr, rb, e, lr, lb);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) f[i] = i == 0 ? (g[0].r - e) + (g[0].b + e) : g[i].r + g[i].b;
+        epi.filled(A, cell, flags);
+      }
+    }
+    ring[hy][hx] = rn;
+  }
+  const CellMoments<R> own = cell_moments<Q, R>(A.ph, f, rr, rb, irho);
+  const bool site = mine && (flags & 1u);
+  const int sites = __syncthreads_count(site);
+  if (GEN && A.ph.phi_field) {
+    long long n = site ? 1 : 0;
+    double removed = site ? (double)e : 0.0;
+    block_sum<P::THREADS>(n, removed);
+    ledger_fold(A.red, n, removed);
+  } else if (tid == 0) {
+    // a scalar flux moves varphi at every site: one 64-bit sum of arrivals (above bit 40) and sites,
+    // order-free, in the place of partials, a fence and a fold by the last CTA
+    const unsigned long long one = 1ull << 40, word = one | (unsigned)sites;
+    const unsigned long long all = atomicAdd(A.red.tally, word) + word;
+    if (all >> 40 == (unsigned long long)gridDim.x * gridDim.y) {
+      const long long c = (long long)(all & (one - 1));
+      const double s = (double)c * A.ph.varphi;
+      DevLedger* led = A.red.ledger;
+      led->evaporated += s;
+      led->last_removed = s;
+      led->site_steps += c;
+      led->last_sites = c;
+      led->steps += 1;
+      *A.red.tally = 0ull;
+    }
+  }
+  if (mine && bits != kNoCell) {
+    R rnb[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const R v = ring[hy + L::cm(i)][hx + L::ca(i)];
+      rnb[i] = (bits >> opp(i)) & 1u ? rn : v;  // a solid neighbour counts as the cell itself
+    }
+    epi.template cell<Q, S>(A, cell, &to, bits, p, si, f, own, rr, rb, irho, lr, lb, flags, rnb);
+  }
+}
+
+template <int S, int TX, int TY>
+static KernelRef patch_ref() {
+  KernelRef k{(const void*)cg_patch_kernel<S, TX, TY, true>, PatchShape<TX, TY>::THREADS};
+  k.tx = TX;
+  k.ty = TY;
+  k.plain = (const void*)cg_patch_kernel<S, TX, TY, false>;
+  k.pdl = 1;
+  return k;
+}
+// Patches of 16 x 8 cells were the fastest or level with the fastest of 8 x 4, 8 x 8, 32 x 4, 16 x 8 and
+// 32 x 8 from 64^2 to 1024^2 (us per step at 64^2 / 256^2 / 1024^2, FP32: 3.3 / 4.6 / 28.1; marched 8.7 /
+// 11.3 / 38.2; F32X 3.4 / 4.9 / 33.0, marched 9.4 / 11.6 / 39.5).  FP64 is held by the FP64 pipe of the
+// SMs it runs on: 8 x 4 until every SM has four of them (64^2: 8.7 against 10.0, marched 19.6), then
+// 16 x 8 (256^2 29.0, marched 43.1; 1024^2 363, marched 371).
+template <int S>
+static KernelRef patch_pick(long long cells) {
+  if (S == ST_F64 && cells <= 152LL * 4 * 32) return patch_ref<S, 8, 4>();
+  return patch_ref<S, 16, 8>();
 }
 
 // The launch record of a pair kernel: the general instantiation and the plain one.
@@ -709,6 +868,7 @@ static KernelRef pair_ref() {
   k.tx = TX;
   k.ty = TY;
   k.plain = plain;
+  k.pdl = 1;
   return k;
 }
 

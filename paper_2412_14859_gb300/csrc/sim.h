@@ -35,6 +35,7 @@ struct cgevap_sim {
   long long part_capacity = 0;
   double* tmp_rn = nullptr;
   int* flag = nullptr;
+  unsigned long long* tally = nullptr;  // Reduce::tally
   int* status = nullptr;  // set by a bounded device-side wait that gave up
   void* staging = nullptr;  // device staging for host imports
   size_t staging_bytes = 0;

@@ -48,4 +48,8 @@ KernelRef step_kernel_f32x(int q, int variant) {
   return {nullptr, 0};
 }
 
+KernelRef patch_kernel_f32(int storage, long long cells) {
+  return storage == ST_F32X ? patch_pick<ST_F32X>(cells) : patch_pick<ST_F32>(cells);
+}
+
 }  // namespace cgevap

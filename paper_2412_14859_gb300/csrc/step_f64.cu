@@ -27,4 +27,6 @@ KernelRef step_kernel_f64(int q, int variant) {
   return {nullptr, 0};
 }
 
+KernelRef patch_kernel_f64(long long cells) { return patch_pick<ST_F64>(cells); }
+
 }  // namespace cgevap
