@@ -29,11 +29,12 @@ struct AdjointTape {
   void* ab = nullptr;              // nstore vec2: the ab part of lambda^{n+1} (then of lambda^n)
   DevLedger* led = nullptr;        // ledger of the recomputed steps (discarded)
   // plan of the forward run, checked by the backward sweep
-  int family = -1, variant = -1, pc = 0;
+  int family = -1, variant = -1, pc = 0, grid_x = 0;
   const void* fwd_fn = nullptr;
   // plan of kernel A
   KernelRef adj{nullptr, 0};
-  int ntx = 1, nty = 1, apc = 1, anchunk = 1;
+  int ntx = 1, nty = 1, apc = 1;
+  dim3 agrid;
   bool recorded = false;
 };
 
@@ -68,12 +69,11 @@ int launch_step_on(cgevap_sim* s, const void* pin, void* pout, const uint8_t* ma
   a.mask_out = mask_out;
   a.red.ledger = ledger;
   void* args[] = {&a};
-  CG_CUDA(s, launch_step(s->kernel, a, dim3(s->ntx * s->nty, s->nchunk), args, s->stream));
+  CG_CUDA(s, launch_step(s->kernel, a, dim3(s->grid_x, s->nchunk), args, s->stream));
   return CGEVAP_OK;
 }
 
-// Kernel A's grid: the step's tiles, planes per chunk chosen as the step planner does
-// (whole waves of resident CTAs against the two extra planes each chunk pulls).
+// Kernel A's grid: the step's tiles, their planes divided as the step planner does.
 int plan_adjoint(cgevap_sim* s, AdjointTape* t) {
   t->adj = adjoint_local_kernel(s->p.q, s->p.storage);
   if (!t->adj.fn) return sim_fail(s, CGEVAP_ERR_UNSUPPORTED, "no adjoint kernel for this configuration");
@@ -86,20 +86,9 @@ int plan_adjoint(cgevap_sim* s, AdjointTape* t) {
   t->nty = (g.nb + t->adj.ty - 1) / t->adj.ty;
   const long long tiles = (long long)t->ntx * t->nty;
   const long long slots = (long long)occ * sms;
-  int best_pc = g.nm;
-  double best = 1e300;
-  for (int pc = 1; pc <= g.nm; ++pc) {
-    const long long nchunk = (g.nm + pc - 1) / pc;
-    if (nchunk > 65535) continue;
-    const double waves = std::ceil((double)(tiles * nchunk) / (double)slots);
-    const double cost = waves * (pc + 2);
-    if (cost < best - 1e-9) {
-      best = cost;
-      best_pc = pc;
-    }
-  }
-  t->apc = best_pc;
-  t->anchunk = (g.nm + best_pc - 1) / best_pc;
+  const MarchPlan mp = plan_march(tiles, g.nm, slots, false);
+  t->apc = mp.pc;
+  t->agrid = dim3((unsigned)tiles, (unsigned)mp.nchunk);
   return CGEVAP_OK;
 }
 
@@ -202,6 +191,7 @@ int cgevap_adjoint_forward(cgevap_sim* s, int nsteps, int ckpt_every, double* de
   t->family = s->family;
   t->variant = s->variant;
   t->pc = s->pc;
+  t->grid_x = s->grid_x;
   t->fwd_fn = s->kernel.fn;
   t->recorded = true;
   return CGEVAP_OK;
@@ -211,7 +201,7 @@ int cgevap_adjoint_backward(cgevap_sim* s, const double* dev_dL_dV, double* dev_
   if (!s || !dev_dL_dphi) return CGEVAP_ERR_ARG;
   AdjointTape* t = s->tape;
   if (!t || !t->recorded) return sim_fail(s, CGEVAP_ERR_ARG, "no recorded forward run");
-  if (t->family != s->family || t->variant != s->variant || t->pc != s->pc || t->fwd_fn != s->kernel.fn)
+  if (t->family != s->family || t->variant != s->variant || t->pc != s->pc || t->grid_x != s->grid_x || t->fwd_fn != s->kernel.fn)
     return sim_fail(s, CGEVAP_ERR_ARG, "the step's tuning changed since cgevap_adjoint_forward");
   CG_CUDA(s, cudaSetDevice(s->device));
   cudaStream_t st = s->stream;
@@ -255,7 +245,7 @@ int cgevap_adjoint_backward(cgevap_sim* s, const double* dev_dL_dV, double* dev_
       o.lam_g = t->lam + (size_t)(lc ^ 1) * t->sb;
       o.aux = t->aux;
       void* args[] = {&a, &o};
-      CG_CUDA(s, cudaLaunchKernel(t->adj.fn, dim3(t->ntx * t->nty, t->anchunk),
+      CG_CUDA(s, cudaLaunchKernel(t->adj.fn, t->agrid,
                                   dim3(t->adj.threads), args, t->adj.smem, st));
       // B1 reads the ab part of lambda^{n+1} no more (kernel A has): it writes lambda^n's
       CG_CUDA(s, launch_adjoint_stencil(ax, t->aux, o.lam_g, t->ab, mn, dev_dL_dphi, inv_sbar,

@@ -364,7 +364,9 @@ __global__ void __launch_bounds__(TX* TY, (S == ST_F64 ? 256 : 384) / (TX * TY))
   constexpr int lam_bytes = Q * TX * TY * (int)sizeof(Vec);
   unsigned char* const lam0 = dyn_smem + PairSmem<Q, S, TX, TY>::BYTES;
   const Epi E{O, lam0 + threadIdx.x * sizeof(Vec), lam0 + lam_bytes};
-  pair_tile<Q, S, TX, TY, true, true>(A, blockIdx.x, blockIdx.y, dyn_smem, n, d, threadIdx.x, E, CtaSync());
+  const int m0 = blockIdx.y * A.pc;
+  pair_tile<Q, S, TX, TY, true, true>(A, blockIdx.x, m0, min(m0 + A.pc, A.g.nm), dyn_smem, n, d, threadIdx.x, E,
+                                      CtaSync());
 }
 
 // (2) one thread per cell.  dLdV: pointer to dL/dV(n+1) (nullptr: 0).  The kernel was bound by its

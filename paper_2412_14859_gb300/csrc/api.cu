@@ -164,8 +164,7 @@ bool tma_supported(const cgevap_sim* s) {
          (s->p.q == 9 || !g.per_b || g.nb >= 4);
 }
 
-// Planes per chunk: balance whole waves of resident CTAs against the two extra planes each
-// chunk pulls (time ~ waves * (pc + 2)); pc_force > 0 overrides.
+// The kernel of a variant and how its planes are divided (plan_march); pc_force > 0 fixes the chunk.
 int plan_launch(cgevap_sim* s, int family, int variant, int pc_force = 0) {
   KernelRef k = family == 1 ? step_tma_f32(s->p.q, variant)
                             : kernel_for(s->p.q, s->p.storage, variant);
@@ -197,21 +196,13 @@ int plan_launch(cgevap_sim* s, int family, int variant, int pc_force = 0) {
   const int nty = patch ? 1 : (nb + t.ty - 1) / t.ty;
   const long long tiles = (long long)ntx * nty;
   const long long slots = (long long)occ * sms;
-  int best_pc = nm;
-  double best = 1e300;
-  for (int pc = 1; pc <= nm; ++pc) {
-    const long long nchunk = (nm + pc - 1) / pc;
-    if (nchunk > 65535) continue;
-    const long long blocks = tiles * nchunk;
-    const double waves = std::ceil((double)blocks / (double)slots);
-    const double cost = waves * (pc + 2);
-    if (cost < best - 1e-9) {
-      best = cost;
-      best_pc = pc;
-    }
+  MarchPlan mp = plan_march(tiles, nm, slots, k.shares != 0);
+  if (pc_force > 0) {
+    mp.pc = pc_force < nm ? pc_force : nm;
+    mp.shares = 0;
   }
-  if (pc_force > 0) best_pc = pc_force < nm ? pc_force : nm;
-  if (patch) best_pc = t.ty;  // rows of a patch
+  if (patch) mp.pc = t.ty;  // rows of a patch
+  if (!mp.shares) mp.nchunk = (nm + mp.pc - 1) / mp.pc;
   if (k.needs_map) {
     const int bh = s->p.q == 19 ? t.ty + 2 : 1;
     for (int h = 0; h < 2; ++h) {
@@ -232,9 +223,10 @@ int plan_launch(cgevap_sim* s, int family, int variant, int pc_force = 0) {
   s->kernel_in = k_in;
   s->ntx = ntx;
   s->nty = nty;
-  s->pc = best_pc;
-  s->nchunk = (nm + best_pc - 1) / best_pc;
-  const long long need = tiles * s->nchunk;
+  s->pc = mp.pc;
+  s->nchunk = mp.nchunk;
+  s->grid_x = mp.shares ? mp.shares : (int)tiles;
+  const long long need = (long long)s->grid_x * s->nchunk;
   if (need > s->part_capacity) {
     if (s->part_removed) cudaFree(s->part_removed);
     if (s->part_sites) cudaFree(s->part_sites);
@@ -296,7 +288,7 @@ int launch_one_step(cgevap_sim* s) {
   StepArgs a = step_args(s);
   void* args[] = {&a, s->tmap[s->cur]};
   const KernelRef& k = s->rc_pairs && s->kernel_in.fn ? s->kernel_in : s->kernel;
-  CG_CUDA(s, launch_step(k, a, dim3(s->ntx * s->nty, s->nchunk), args, s->stream));
+  CG_CUDA(s, launch_step(k, a, dim3(s->grid_x, s->nchunk), args, s->stream));
   s->cur ^= 1;
   s->rc_pairs = 0;
   return CGEVAP_OK;
@@ -837,7 +829,10 @@ int cgevap_get_tuning(const cgevap_sim* s, int* family, int* variant, int* plane
   if (!s) return CGEVAP_ERR_ARG;
   if (family) *family = s->family;
   if (variant) *variant = s->variant;
-  if (planes_per_chunk) *planes_per_chunk = s->pc;
+  // an even division among the CTAs: the planes of the largest share
+  if (planes_per_chunk)
+    *planes_per_chunk = s->pc > 0 ? s->pc
+                                  : (int)(((long long)s->ntx * s->nty * s->geom.nm + s->grid_x - 1) / s->grid_x);
   return CGEVAP_OK;
 }
 

@@ -122,7 +122,8 @@ struct StepArgs {
   Physics ph;
   Reduce red;
   int ntx, nty;                  // tiles along a and b
-  int pc;                        // planes per chunk along m
+  int pc;                        // planes per chunk along m; 0: the tiles' planes, tile after tile,
+                                 // are divided evenly among the CTAs (pair storages)
   const void* pin;               // state read (post-recoloring populations of the last step)
   void* pout;                    // state written
   const uint8_t* mask_in;        // site bytes of the last step

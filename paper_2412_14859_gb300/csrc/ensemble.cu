@@ -168,10 +168,11 @@ __global__ void __launch_bounds__(kEnsThreads, MODE == kEnsF32 || MODE == kEnsF3
         if (tid == 0) set_buffers(args[0], it.x, step);
         __syncthreads();
         const bool f64 = MODE == kEnsF64 || (MODE == kEnsMixed && E.members[it.x].storage == ST_F64);
+        const int m0 = it.z * args[0].pc;
         if (MODE != kEnsF64 && !f64)
-          pair_tile<19, S32, 32, kEnsTy, true, GEN>(args[0], it.y, it.z, smem, n, d, tid, PairStep<GEN>(), CtaSync());
+          pair_tile<19, S32, 32, kEnsTy, true, GEN>(args[0], it.y, m0, m0 + it.w, smem, n, d, tid, PairStep<GEN>(), CtaSync());
         else if (MODE == kEnsF64 || MODE == kEnsMixed)
-          pair_tile<19, ST_F64, 32, kEnsTy, false, GEN>(args[0], it.y, it.z, smem, n, d, tid, PairStep<GEN>(), CtaSync());
+          pair_tile<19, ST_F64, 32, kEnsTy, false, GEN>(args[0], it.y, m0, m0 + it.w, smem, n, d, tid, PairStep<GEN>(), CtaSync());
         block_sum<NT>(n, d);
         if (tid == 0) {
           pr[w] = d;
@@ -192,10 +193,11 @@ __global__ void __launch_bounds__(kEnsThreads, MODE == kEnsF32 || MODE == kEnsF3
           sync.wait();
           if (gtid == 0) set_buffers(A, it.x, step);
           sync.wait();
+          const int m0 = it.z * A.pc;
           if (MODE != kEnsF64 && !f64)
-            pair_tile<9, S32, GT, 1, true, GEN>(A, it.y, it.z, gs, n, d, gtid, PairStep<GEN>(), sync);
+            pair_tile<9, S32, GT, 1, true, GEN>(A, it.y, m0, m0 + it.w, gs, n, d, gtid, PairStep<GEN>(), sync);
           else if (MODE == kEnsF64 || MODE == kEnsMixed)
-            pair_tile<9, ST_F64, GT, 1, false, GEN>(A, it.y, it.z, gs, n, d, gtid, PairStep<GEN>(), sync);
+            pair_tile<9, ST_F64, GT, 1, false, GEN>(A, it.y, m0, m0 + it.w, gs, n, d, gtid, PairStep<GEN>(), sync);
         }
         // per-group sums: warp shuffles, then the group's warps in shared memory
 #pragma unroll

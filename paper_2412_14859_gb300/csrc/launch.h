@@ -29,6 +29,7 @@ struct KernelRef {
   int smem = 0;       // dynamic shared memory bytes
   int tx = 0, ty = 0; // tile shape (0: take it from tile_cfg)
   int needs_map = 0;  // 1: second kernel argument is the TMA tensor map of the input state
+  int shares = 0;               // 1: can divide the tiles' planes evenly (StepArgs::pc = 0)
   int pdl = 0;                  // 1: may be launched ahead of its predecessor's end (it waits itself)
   const void* plain = nullptr;  // the same step without links, site bytes read or a flux field
 };
@@ -49,6 +50,33 @@ inline cudaError_t launch_step(const KernelRef& k, const StepArgs& a, dim3 grid,
   cfg.attrs = &ahead;
   cfg.numAttrs = k.pdl ? 1u : 0u;
   return cudaLaunchKernelExC(&cfg, step_fn(k, a), args);
+}
+// How a tiled kernel's planes are divided among `slots` resident CTAs: in chunks of pc planes (the
+// time is about waves x (pc + 2) planes, the two extra ones pulled at each chunk's ends), or, pc = 0
+// and `shares` CTAs, evenly across tile ends (share + 2 planes per piece of a tile; for_planes).
+struct MarchPlan {
+  int pc, nchunk, shares;
+};
+inline MarchPlan plan_march(long long tiles, int nm, long long slots, bool can_share) {
+  MarchPlan best{nm, 1, 0};
+  double cost = 1e300;
+  for (int pc = 1; pc <= nm; ++pc) {
+    const long long nchunk = (nm + pc - 1) / pc;
+    if (nchunk > 65535) continue;
+    const long long waves = (tiles * nchunk + slots - 1) / slots;
+    const double c = (double)waves * (pc + 2);
+    if (c < cost - 1e-9) {
+      cost = c;
+      best = MarchPlan{pc, (int)nchunk, 0};
+    }
+  }
+  if (can_share && tiles * nm > slots) {
+    const long long share = (tiles * nm + slots - 1) / slots;
+    const long long pieces = nm % share == 0 ? 1 : (share - 1) / nm + 2;
+    // by more than the model's own error
+    if ((double)(share + 2 * pieces) < 0.98 * cost) best = MarchPlan{0, 1, (int)slots};
+  }
+  return best;
 }
 KernelRef step_kernel_f64(int q, int variant);
 KernelRef step_kernel_f32(int q, int variant);

@@ -46,7 +46,8 @@ struct cgevap_sim {
   cgevap::KernelRef kernel_in{nullptr, 0};  // F32RC: the same step reading FP32 pairs
   int rc_pairs = 1;  // F32RC: state[cur] holds FP32 pairs (created or imported, not yet stepped)
   alignas(64) unsigned char tmap[2][128];  // TMA tensor maps of state[0] and state[1]
-  int ntx = 1, nty = 1, pc = 1, nchunk = 1;
+  int ntx = 1, nty = 1, pc = 1, nchunk = 1;  // pc = 0: even shares (StepArgs::pc)
+  int grid_x = 1;                            // CTAs along grid x: tiles, or even shares
   cgevap::AdjointTape* tape = nullptr;  // checkpoints of cgevap_adjoint_forward (adjoint.cu)
   double* vol_part = nullptr;           // cgevap_volume scratch: kVolumeBlocks partials
   unsigned int* vol_done = nullptr;     // and its arrival counter
