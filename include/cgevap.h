@@ -275,7 +275,9 @@ CGEVAP_API int cgevap_calibrate_threshold(const cgevap_params* p, double phi, do
  * register-pipelined kernel, measured faster), 0 the
  * register-pipelined kernel (every storage, any nx), 1 the bulk-copy pipelined kernel (FP32
  * storage and even nx); variant picks a tile shape / pipeline depth of that family (0 = default);
- * planes_per_chunk > 0 fixes how many planes one CTA marches through (0 = planner).  All
+ * planes_per_chunk > 0 fixes how many planes one CTA marches through (0 = planner: chunks, or for
+ * FP64 an even share of all tiles' planes per CTA; D2Q9 F64 / F32 / F32X with variant 0 then takes
+ * patches of rows instead of marching).  All
  * choices compute the same result; they differ in speed only.  Errors: ARG, UNSUPPORTED. */
 CGEVAP_API int cgevap_tune(cgevap_sim* sim, int family, int variant, int planes_per_chunk);
 /* The current choice of cgevap_tune (any output pointer may be NULL). */

@@ -196,7 +196,8 @@ int plan_launch(cgevap_sim* s, int family, int variant, int pc_force = 0) {
   const int nty = patch ? 1 : (nb + t.ty - 1) / t.ty;
   const long long tiles = (long long)ntx * nty;
   const long long slots = (long long)occ * sms;
-  MarchPlan mp = plan_march(tiles, nm, slots, k.shares != 0);
+  MarchPlan mp = plan_march(tiles, nm, slots, k.shares != 0,
+                            s->p.storage == CGEVAP_F16DEV || s->p.storage == CGEVAP_BF16DEV ? 0.0 : kExtraPlanes);
   if (pc_force > 0) {
     mp.pc = pc_force < nm ? pc_force : nm;
     mp.shares = 0;
