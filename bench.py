@@ -36,7 +36,7 @@ sys.path.insert(0, ROOT)
 
 METRIC = "MLUPS & % of HBM roofline, CG-LBM+evaporation step; mixed vs FP64 at stated error"
 UNIT = "MLUPS"
-KERNEL_SOURCES = ["lattice.cuh", "common.cuh", "step_kernel.cuh"]
+KERNEL_SOURCES = ["lattice.cuh", "common.cuh", "step_kernel.cuh", "pair_tile.cuh"]
 
 
 def parse():
