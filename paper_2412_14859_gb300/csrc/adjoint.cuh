@@ -212,6 +212,38 @@ __device__ __forceinline__ void collide_adjoint(const Physics& ph, const CellMom
   });
 }
 
+// The auxiliary fields of kernel A: per cell (dL/dF_a, dL/dF_b, dL/dF_m, d rho^N/d rho_r) side by
+// side, so that B1 takes a neighbour's gradient in one 16-byte load (two for FP64), and after those
+// nstore cells a plane of d rho^N/d rho_b (a fit iteration of 32 steps on the full cap 72.56 ms with
+// five planes, 72.26 so; at six or four CTAs per SM instead of eight 72.65 and 73.74).
+template <class R>
+struct AuxCell;
+template <>
+struct AuxCell<float> {
+  float a, b, m, dr;
+  static __device__ __forceinline__ AuxCell load(const void* aux, int si) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(aux) + si);
+    return {v.x, v.y, v.z, v.w};
+  }
+  static __device__ __forceinline__ void store(void* aux, int si, const float (&F)[3], float dr) {
+    reinterpret_cast<float4*>(aux)[si] = make_float4(F[0], F[1], F[2], dr);
+  }
+};
+template <>
+struct AuxCell<double> {
+  double a, b, m, dr;
+  static __device__ __forceinline__ AuxCell load(const void* aux, int si) {
+    const double2* p = reinterpret_cast<const double2*>(aux) + 2 * (size_t)si;
+    const double2 v = __ldg(p), w = __ldg(p + 1);
+    return {v.x, v.y, w.x, w.y};
+  }
+  static __device__ __forceinline__ void store(void* aux, int si, const double (&F)[3], double dr) {
+    double2* p = reinterpret_cast<double2*>(aux) + 2 * (size_t)si;
+    p[0] = make_double2(F[0], F[1]);
+    p[1] = make_double2(F[2], dr);
+  }
+};
+
 // lg_i goes where the pull read g_i from: slot i of x - c_i, or slot opp(i) of x for a bounced link
 // (element index in 32 bits: a state holds Q nstore < 2^31 vec2).
 template <int Q, class R, class Vec>
@@ -341,12 +373,8 @@ struct AdjointEpilogue {
     R Fa, Fb, Fm;
     colour_gradient<Q, R>(rnb, Fa, Fb, Fm);
     collide_adjoint<Q, R>(A.ph, c, f, irho, Fa, Fb, Fm, lam_at, lg_out, lF);
-    R* ax = reinterpret_cast<R*>(o.aux);
-    ax[si] = lF[0];
-    ax[(size_t)ns + si] = lF[1];
-    ax[2 * (size_t)ns + si] = lF[2];
-    ax[3 * (size_t)ns + si] = R(2) * rb * irho * irho;   // d rho^N / d rho_r
-    ax[4 * (size_t)ns + si] = -R(2) * rr * irho * irho;  // d rho^N / d rho_b
+    AuxCell<R>::store(o.aux, si, lF, R(2) * rb * irho * irho);  // ... and d rho^N / d rho_r
+    reinterpret_cast<R*>(o.aux)[4 * ns + si] = -R(2) * rr * irho * irho;  // d rho^N / d rho_b
   }
 };
 
@@ -399,15 +427,19 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 8 : 5)  // FP32: 32 regi
       const int4 to = make_int4(sl.dxm, sl.dxp, sl.dym, sl.dyp);
       const int si = sidx(G, a, b, m);
       const int ns = G.nstore;  // 5 ns < Q nstore < 2^31
-      const R oa = aux[si], ob = aux[ns + si], om = aux[2 * ns + si];
+      const AuxCell<R> own = AuxCell<R>::load(aux, si);
       R mu = w0;
+      auto along = [](int i, const AuxCell<R>& F) {  // F . c_i
+        R t = R(0);
+        if (L::ca(i)) t += R(L::ca(i)) * F.a;
+        if (L::cb(i)) t += R(L::cb(i)) * F.b;
+        if (L::cm(i)) t += R(L::cm(i)) * F.m;
+        return t;
+      };
       auto from = [&](int i) {  // F of x = y - c_i used rho^N(y) with weight 3 W_i c_i
         const int src = pull_source<L>(to, po.dm_lo, po.dm_hi, si, i);
-        R t = R(0);
-        if (L::ca(i)) t += R(L::ca(i)) * __ldg(aux + src);
-        if (L::cb(i)) t += R(L::cb(i)) * __ldg(aux + (ns + src));
-        if (L::cm(i)) t += R(L::cm(i)) * __ldg(aux + (2 * ns + src));
-        return t;
+        const AuxCell<R> F = AuxCell<R>::load(aux, src);
+        return along(i, F);
       };
       if (bits == 0) {
 #pragma unroll
@@ -418,12 +450,12 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 8 : 5)  // FP32: 32 regi
           R t = R(0);
           if (!((bits >> i) & 1u)) t = from(i);  // x = y - c_i is fluid
           if ((bits >> opp(i)) & 1u)  // y + c_i is solid: y's own F used rho^N(y) in its place
-            t += R(L::ca(i)) * oa + R(L::cb(i)) * ob + R(L::cm(i)) * om;
+            t += along(i, own);
           mu += R(3.0 * L::W(i)) * t;
         }
       }
       Vec v;
-      v.x = mu * aux[3 * ns + si];
+      v.x = mu * own.dr;
       v.y = mu * aux[4 * ns + si];
       reinterpret_cast<Vec*>(ab)[si] = v;
       if (mask[cell] & 1u) {  // Eq. (exchange): d g_0^r / d phi = -1/S-bar, d g_0^b / d phi = +1/S-bar

@@ -145,8 +145,8 @@ cudaError_t launch_heated_flux(const AuxArgs& a, const void* state, double* part
 
 // Adjoint sweep (adjoint_kernels.cu).  The local kernel (kernel A) takes (StepArgs, AdjointOut)
 // and runs on the step's tile grid; F64 / F32 storage only.
-// Auxiliary per-cell fields of the sweep, planes of nstore reals in the storage layout:
-// dL/dF_a, dL/dF_b, dL/dF_m, d rho^N/d rho_r, d rho^N/d rho_b.
+// Auxiliary per-cell fields of the sweep, five reals for each of nstore cells (AuxCell): dL/dF_a,
+// dL/dF_b, dL/dF_m and d rho^N/d rho_r side by side, then the plane of d rho^N/d rho_b.
 constexpr int kAdjAuxPlanes = 5;
 struct AdjointOut {
   const void* lam_in;  // the lg part of lambda^{n+1} = dL/df^{n+1}, pushed by the previous
