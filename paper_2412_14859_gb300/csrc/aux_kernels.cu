@@ -144,7 +144,8 @@ __global__ void k_macros(Geom g, Physics ph, const void* state, double* rr_out, 
     double fr[Q], fb[Q];
     load_cell<Q, S>(state, g, cell, fr, fb, ph);
     // bound by the FP64 rate: momenta from the differences of opposite directions, no products with
-    // c, one division a cell
+    // c.  The quotients are divisions: a product with 1 / rho takes one rounding more, and rho^N of a
+    // cell of one colour is then not +-1
     double rr = fr[0], rb = fb[0], ja = 0, jb = 0, jm = 0;
 #pragma unroll
     for (int i = 1; i < Q; i += 2) {
@@ -158,16 +159,15 @@ __global__ void k_macros(Geom g, Physics ph, const void* state, double* rr_out, 
       }
     }
     const double rho = rr + rb;
-    const double irho = 1.0 / rho;
     const bool solid = cell_solid(g, cell) || !(rho > 0.0);
     if (rr_out) rr_out[cell] = solid ? 0.0 : rr;
     if (rb_out) rb_out[cell] = solid ? 0.0 : rb;
-    if (rn_out) rn_out[cell] = solid ? 0.0 : (rr - rb) * irho;
+    if (rn_out) rn_out[cell] = solid ? 0.0 : (rr - rb) / rho;
     if (u_out) {
       // (a, b, m) -> (x, y, z): 3D (x, y, z); 2D (x, -, y)
-      const double ux = solid ? 0.0 : ja * irho;
-      const double uy = solid ? 0.0 : (L::D3 ? jb : jm) * irho;
-      const double uz = solid ? 0.0 : (L::D3 ? jm : 0.0) * irho;
+      const double ux = solid ? 0.0 : ja / rho;
+      const double uy = solid ? 0.0 : (L::D3 ? jb : jm) / rho;
+      const double uz = solid ? 0.0 : (L::D3 ? jm : 0.0) / rho;
       u_out[cell] = ux;
       u_out[(size_t)g.ncell + cell] = uy;
       u_out[2 * (size_t)g.ncell + cell] = uz;
