@@ -280,7 +280,9 @@ CGEVAP_API int cgevap_calibrate_threshold(const cgevap_params* p, double phi, do
  * patches of rows instead of marching).  All
  * choices compute the same result; they differ in speed only.  Errors: ARG, UNSUPPORTED. */
 CGEVAP_API int cgevap_tune(cgevap_sim* sim, int family, int variant, int planes_per_chunk);
-/* The current choice of cgevap_tune (any output pointer may be NULL). */
+/* The current choice of cgevap_tune (any output pointer may be NULL).  planes_per_chunk is the length
+ * in use, the planner's or a fixed one, and 0 where the planner divides the lattice otherwise (even
+ * shares, patches); cgevap_tune with the three values keeps the plan as it is. */
 CGEVAP_API int cgevap_get_tuning(const cgevap_sim* sim, int* family, int* variant,
                                  int* planes_per_chunk);
 

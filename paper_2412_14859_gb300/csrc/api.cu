@@ -227,6 +227,7 @@ int plan_launch(cgevap_sim* s, int family, int variant, int pc_force = 0) {
   s->pc = mp.pc;
   s->nchunk = mp.nchunk;
   s->grid_x = mp.shares ? mp.shares : (int)tiles;
+  s->chunked = !patch && !mp.shares;
   const long long need = (long long)s->grid_x * s->nchunk;
   if (need > s->part_capacity) {
     if (s->part_removed) cudaFree(s->part_removed);
@@ -830,10 +831,8 @@ int cgevap_get_tuning(const cgevap_sim* s, int* family, int* variant, int* plane
   if (!s) return CGEVAP_ERR_ARG;
   if (family) *family = s->family;
   if (variant) *variant = s->variant;
-  // an even division among the CTAs: the planes of the largest share
-  if (planes_per_chunk)
-    *planes_per_chunk = s->pc > 0 ? s->pc
-                                  : (int)(((long long)s->ntx * s->nty * s->geom.nm + s->grid_x - 1) / s->grid_x);
+  // 0 (cgevap_tune: the planner's choice) for patches and even shares, which no chunk length selects
+  if (planes_per_chunk) *planes_per_chunk = s->chunked ? s->pc : 0;
   return CGEVAP_OK;
 }
 

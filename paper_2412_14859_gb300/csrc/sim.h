@@ -48,6 +48,7 @@ struct cgevap_sim {
   alignas(64) unsigned char tmap[2][128];  // TMA tensor maps of state[0] and state[1]
   int ntx = 1, nty = 1, pc = 1, nchunk = 1;  // pc = 0: even shares (StepArgs::pc)
   int grid_x = 1;                            // CTAs along grid x: tiles, or even shares
+  bool chunked = true;                       // the plan is chunks of pc planes (not patches, not shares)
   cgevap::AdjointTape* tape = nullptr;  // checkpoints of cgevap_adjoint_forward (adjoint.cu)
   double* vol_part = nullptr;           // cgevap_volume scratch: kVolumeBlocks partials
   unsigned int* vol_done = nullptr;     // and its arrival counter
