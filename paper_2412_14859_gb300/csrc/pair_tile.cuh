@@ -128,18 +128,25 @@ __device__ __forceinline__ void pull_pairs(const void* pin, int ns, int4 to, int
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float recip_density(float x) { return __frcp_rn(x); }
-// FP64: the hardware's approximation e_0 = 1 - x y (about 2^-20) and one third-order
-// Newton-Householder step, y (1 + e + e^2): e_0^3 is below the rounding of the last product.
+// FP64: from the hardware's approximation y one step of Householder's iteration of third order for
+// x^-1: with e = 1 - x y, 1 / x = y / (1 - e) = y (1 + e + e^2) + O(y e^3).  y is good to about 2^-20,
+// so e^3 and the rounding of e + e^2 lie below the rounding of the last product, and the result is
+// within 1.1 half-ulps of 1 / x.  The approximation takes and gives no subnormals; where x or 1 / x is
+// one (and for 0, infinity and NaN) the division.
+static __device__ __noinline__ double divide_one(double x) { return 1.0 / x; }  // inlined, a step took 1.2 % longer
 __device__ __forceinline__ double recip_density(double x) {
+  const unsigned h = (unsigned)__double2hiint(x) & 0x7fffffffu;
+  if (h - 0x00100000u >= 0x7fd00000u - 0x00100000u) return divide_one(x);  // not 2^-1022 <= |x| < 2^1022
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double e = fma(-x, y, 1.0);
   return fma(y, fma(e, e, e), y);
 }
-// |F| and 1 / |F| from F2 = |F|^2 > 0.  FP64: the same third-order step for x^(-1/2),
-// y (1 + e/2 + 3 e^2/8) with e = 1 - F2 y^2; outside the range the approximation holds for, the
-// square root and the division (GB300 issues an FP64 instruction every 16 cycles a warp: 7 of
-// them here against about 25).
+// |F| and 1 / |F| from F2 = |F|^2 > 0.  FP64: the iteration of third order for x^(-1/2): with
+// e = 1 - F2 y^2, F2^(-1/2) = y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2/8) + O(y e^3), within 1.6 half-ulps
+// (half of the rounding of F2 y reaches the result), and |F| = F2 / |F| within 2.6.  Outside the range
+// in which F2 and its root are far from subnormals, the square root and the division (GB300 issues an
+// FP64 instruction every 16 cycles a warp: 7 of them here against about 25).
 __device__ __forceinline__ void norm_of(float F2, float& Fn, float& iFn) {
   iFn = rsqrtf(F2);
   Fn = mul_rn(F2, iFn);
