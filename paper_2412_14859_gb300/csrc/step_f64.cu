@@ -13,7 +13,7 @@ KernelRef step_kernel_f64(int q, int variant) {
   if (q == 19) {
     switch (variant) {
       case 0: return reg_ref<19, 16, 8, 2>();
-      case 1: return reg_ref<19, 32, 8, 1>();
+      case 1: return reg_ref<19, 32, 8, 1>();  // 240 registers a thread; variant 3: 128, two CTAs per SM
       case 2: return reg_ref<19, 16, 16, 1>();
       case 3: return reg_ref<19, 32, 8, 2>();
       case 4: return reg_ref<19, 32, 4, 2>();

@@ -132,10 +132,6 @@ __device__ __forceinline__ void async_wait_all() { asm volatile("cp.async.wait_a
 template <class R>
 __device__ __forceinline__ R recip(R x);
 template <>
-__device__ __forceinline__ double recip<double>(double x) {
-  return 1.0 / x;
-}
-template <>
 __device__ __forceinline__ float recip<float>(float x) {
   return __frcp_rn(x);
 }
@@ -178,21 +174,11 @@ __device__ __forceinline__ typename Storage<S>::real site_exchange(
     typename Storage<S>::real& rr, typename Storage<S>::real& rb, typename Storage<S>::real& e,
     uint32_t& flags, typename Storage<S>::real& irho) {
   using R = typename Storage<S>::real;
-  R sr = R(0), sb = R(0);
-  if constexpr (std::is_same<R, float>::value) {  // both components in packed FP32
-    float2 acc = make_float2(0.0f, 0.0f);
+  static_assert(std::is_same<R, float>::value, "FP64 marches in pair_tile.cuh");
+  float2 acc = make_float2(0.0f, 0.0f);  // both components in packed FP32
 #pragma unroll
-    for (int i = 0; i < Q; ++i) acc = __fadd2_rn(acc, make_float2(g[i].r, g[i].b));
-    sr = acc.x;
-    sb = acc.y;
-  } else {
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      sr += g[i].r;
-      sb += g[i].b;
-    }
-  }
-  const R rn = exchange_from_sums<S>(A, cell, sr, sb, rr, rb, e, flags, irho);
+  for (int i = 0; i < Q; ++i) acc = __fadd2_rn(acc, make_float2(g[i].r, g[i].b));
+  const R rn = exchange_from_sums<S>(A, cell, acc.x, acc.y, rr, rb, e, flags, irho);
   g[0].r -= e;
   g[0].b += e;
   return rn;
@@ -687,25 +673,14 @@ __device__ __forceinline__ void collide_store(const StepArgs& A, int si, int nim
     const R odd = R(3) * rwc[c] * cu;
     const R pert = fma(kw[c], pc * pc, -kc[c]);  // Eq. (perturb), even in c
     const R kp = kr[c] * pc;                     // Eq. (recolor) term, odd in c
-    R fi, fj, fri, frj;
-    if constexpr (std::is_same<R, float>::value) {
-      // both directions of the pair in packed FP32 (same roundings as the scalar form)
-      const float2 fv = make_float2(f[i], f[j]);
-      const float2 m1 = make_float2(-1.0f, -1.0f);
-      const float2 feq = __fadd2_rn(make_float2(even, even), make_float2(odd, -odd));
-      float2 post = __ffma2_rn(make_float2(itau, itau), __ffma2_rn(fv, m1, feq), fv);
-      post = __fadd2_rn(post, make_float2(pert, pert));
-      const float2 fr = __ffma2_rn(make_float2(wr, wr), post, make_float2(kp, -kp));
-      fi = post.x;
-      fj = post.y;
-      fri = fr.x;
-      frj = fr.y;
-    } else {
-      fi = fma(itau, (even + odd) - f[i], f[i]) + pert;  // Eq. (collision) + (perturb)
-      fj = fma(itau, (even - odd) - f[j], f[j]) + pert;
-      fri = fma(wr, fi, kp);
-      frj = fma(wr, fj, -kp);
-    }
+    // both directions of the pair in packed FP32
+    const float2 fv = make_float2(f[i], f[j]);
+    const float2 m1 = make_float2(-1.0f, -1.0f);
+    const float2 feq = __fadd2_rn(make_float2(even, even), make_float2(odd, -odd));
+    float2 post = __ffma2_rn(make_float2(itau, itau), __ffma2_rn(fv, m1, feq), fv);
+    post = __fadd2_rn(post, make_float2(pert, pert));  // Eq. (collision) + (perturb)
+    const float2 fr = __ffma2_rn(make_float2(wr, wr), post, make_float2(kp, -kp));
+    const R fi = post.x, fj = post.y, fri = fr.x, frj = fr.y;
     if constexpr (Storage<S>::rc16) {
       // encode f - r_i Rf (s scaled) in 16 bits, decode as a reader will, and split the decoded
       // values with this cell's record exactly as the readers will split them
