@@ -790,6 +790,7 @@ def run_ours(args, d: Dist):
                      "peak_source": peak_src,
                      "algorithmic_bytes_per_update": H["bytes_per_update"],
                      "kernel": ("cg_step_tma_kernel" if H["tuning"]["family"] == 1 else
+                                "cg_pair_kernel" if head in ("f64", "f32", "f32x") else
                                 "cg_step_kernel") + " (fused step), tuning %s" % H["tuning"]},
         "variants": variants,
         "gpu_launches": args.steps,
